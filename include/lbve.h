@@ -82,12 +82,12 @@ typedef enum { LBVE_F64 = 0, LBVE_F32 = 1, LBVE_F16_SHIFTED = 2, LBVE_BF16_SHIFT
 
 /* Kernel schedule: two kernels per step (LB, then FV), or one fused kernel per step.
  * SPLIT: the per-cell stream-collide (the LB half, Eqs. (lb), (guo), (force), (ubb)) and
- * the tiled stress update.  PIPELINED: the split schedule with the row-pipelined
+ * the tiled stress update (FP64: the per-cell stress update).  PIPELINED: the split schedule with the row-pipelined
  * stream-collide and the two-cell stress update wherever the grid allows them (see
  * lbve_stream_collide_kernel, lbve_stress_kernel).  AUTO: PIPELINED for large grids (the
  * row pipeline from 2^22 cells in FP32 and 16-bit storage, the two-cell stress update
- * from 2^21, where they were measured faster on GB300), SPLIT below.  All three give
- * bitwise the same results. */
+ * from 2^21, where they were measured faster on GB300), SPLIT below, with a per-cell
+ * stress update below 3 * 2^18 cells.  All three give bitwise the same results. */
 #define LBVE_SCHED_AUTO 0
 #define LBVE_SCHED_SPLIT 1
 #define LBVE_SCHED_FUSED 2
@@ -283,7 +283,8 @@ int lbve_stream_collide_kernel(const lbve_ctx *ctx);
  * FP32, FP16 and BF16 storage when the solve uses the method's own update (flux and
  * source on; no CTU, tau div u, Giesekus or FENE-P term), nx is a multiple of 4 and the
  * arrays are 16-byte aligned (always with the library's own allocations).
- * LBVE_FV_TILES: 32 x 8 columns, one cell per thread.  Results are bitwise equal.  -1 for
+ * LBVE_FV_TILES: one cell per thread, in 32 x 8 columns or, on small grids and in FP64,
+ * cell by cell.  Results are bitwise equal.  -1 for
  * NULL.
  */
 #define LBVE_FV_TILES 0
@@ -370,8 +371,8 @@ lbve_status lbve_read_kernel_times(lbve_ctx *ctx, double ms[LBVE_KT_COUNT], long
  *          resting walls.  Momentum-exchange forces are not computed by this call.
  *          The call sets the stress of every non-fluid cell to zero in tau_a and tau_b
  *          (a solid cell carries no stress; the stress update relies on it).
- * Schedule: always the split kernels (the per-cell stream-collide and the tiled stress
- * update).  p->schedule must be LBVE_SCHED_AUTO or LBVE_SCHED_SPLIT (LBVE_SCHED_FUSED and
+ * Schedule: always the split kernels (the per-cell stream-collide, and the stress kernel
+ * the schedule takes on a grid of this size).  p->schedule must be LBVE_SCHED_AUTO or LBVE_SCHED_SPLIT (LBVE_SCHED_FUSED and
  * LBVE_SCHED_PIPELINED are rejected with EINVAL); p->block_x is honoured as
  * by lbve_create, but schedules recorded by lbve_autotune are not applied and the stress
  * kernel takes its default z-chunk.  None of these choices changes a result.

@@ -36,6 +36,21 @@ constexpr int lb_min_blocks() {
 #define LBVE_LBB_MIN_BLOCKS 7   // serving mix's pool step measured 1.201 ms at 7, 1.217 at 8)
 #endif
 
+// Division of a 32-bit dividend below 2^31 by a fixed divisor (T. Granlund and
+// P. L. Montgomery, "Division by invariant integers using multiplication", 1994):
+// q = (mulhi(m, n) + n) >> s with s = ceil(log2 d), m = floor(2^32 (2^s - d) / d) + 1.
+struct FastDiv {
+    unsigned m, s;
+    __host__ __device__ static FastDiv of(unsigned d) {
+        FastDiv f;
+        f.s = 0;
+        while ((1ull << f.s) < d) ++f.s;
+        f.m = (unsigned)((((1ull << f.s) - d) << 32) / d + 1ull);
+        return f;
+    }
+    __device__ __forceinline__ unsigned div(unsigned n) const { return (__umulhi(m, n) + n) >> s; }
+};
+
 template <class S>
 struct KArgs {
     using R = typename Store<S>::R;
@@ -53,6 +68,8 @@ struct KArgs {
     unsigned *bad;  // instability flag (mapped host word) or nullptr
     int zlo, zhi;   // planes the step kernels compute
     unsigned key_base;  // added to the cell index in rounding keys (a z-slab: its global offset)
+    unsigned lin;       // cells of the computed planes (per-cell kernels in memory order)
+    FastDiv dnx, dny;   // division by nx, ny
     // per-direction / per-component bases (f + i np, tau + c np, u_out + k np, u_in + k np,
     // tau_out + c np), so that an address is one multiply-add of a 32-bit cell index; set
     // by link_dirs
@@ -231,42 +248,46 @@ __device__ __forceinline__ void lb_core(const KArgs<S> &a, const Cell &cl, unsig
     lb_core_f<S, PAR>(a, cl, r, mask, tr, tn, f);
 }
 
-// Velocity / stress / boundary-velocity accessors of the face neighbours in global memory.
-template <class R>
+// Velocity / stress / boundary-velocity accessors of the face neighbours in global memory
+// (kernel parameters: per-component bases, one multiply-add per address).
+template <class S>
 struct GlobalNb {
-    const Geo &g;
-    const Phys<R> &ph;
+    using R = typename Store<S>::R;
+    const KArgs<S> &a;
     const Cell &cl;
-    const R *tau;
-    const R *u;
-    const uint8_t *flag;
-    const PartDev *parts;
     __device__ __forceinline__ unsigned at(int l) const {
         const int k = l >> 1, s = (l & 1) ? -1 : 1;
         return cl.idx(k == 0 ? s : 0, k == 1 ? s : 0, k == 2 ? s : 0);
     }
-    __device__ __forceinline__ R u_(int l, int j) const { return u[j * (size_t)g.np + at(l)]; }
-    __device__ __forceinline__ R tau_(int l, int c) const { return tau[c * (size_t)g.np + at(l)]; }
-    __device__ __forceinline__ void ub_(int l, R out[3]) const {
+    __device__ __forceinline__ R u(int l, int j) const { return a.uiq[j][at(l)]; }
+    __device__ __forceinline__ R tau(int l, int c) const { return a.tq[c][at(l)]; }
+    __device__ __forceinline__ void ub(int l, R out[3]) const {
         const int k = l >> 1, s = (l & 1) ? -1 : 1;
         const int dx = k == 0 ? s : 0, dy = k == 1 ? s : 0, dz = k == 2 ? s : 0;
-        boundary_velocity_fast<R>(g, ph, parts, flag[at(l)], cl.X(dx), cl.Y(dy), cl.Z(dz), out);
+        boundary_velocity_fast<R>(a.g, a.ph, a.parts, a.flag[at(l)], cl.X(dx), cl.Y(dy), cl.Z(dz), out);
     }
 };
-template <class R>
-struct NbAdapter {  // gives GlobalNb the u / tau / ub interface fv_core expects
-    const GlobalNb<R> &n;
-    __device__ __forceinline__ R u(int l, int j) const { return n.u_(l, j); }
-    __device__ __forceinline__ R tau(int l, int c) const { return n.tau_(l, c); }
-    __device__ __forceinline__ void ub(int l, R out[3]) const { n.ub_(l, out); }
-};
 
-// Launch shape of the per-cell kernels: blockDim (bx, by), grid (nx/bx, ny/by, nz).
-__device__ __forceinline__ bool cell_of_thread(const Geo &g, int &x, int &y, int &z) {
+// Cell of a thread of the per-cell kernels: blocks of x-y tiles (blockDim (bx, by), grid
+// (nx/bx, ny/by, nz)), or, where tiles would leave lanes idle (83 cells on 64-wide blocks:
+// 65 % of the lanes used), the cells of the computed planes in memory order (LIN: a.lin of
+// them, one-dimensional grid; a build of its own, the choice at run time spilled registers
+// in the stream-collide).
+template <class S, bool LIN>
+__device__ __forceinline__ bool cell_of_thread(const KArgs<S> &a, int &x, int &y, int &z) {
+    if constexpr (LIN) {
+        const unsigned r = blockIdx.x * blockDim.x + threadIdx.x;
+        if (r >= a.lin) return false;
+        const unsigned row = a.dnx.div(r), pl = a.dny.div(row);
+        x = (int)(r - row * (unsigned)a.g.nx);
+        y = (int)(row - pl * (unsigned)a.g.ny);
+        z = (int)pl + a.zlo;
+        return true;
+    }
     x = blockIdx.x * blockDim.x + threadIdx.x;
     y = blockIdx.y * blockDim.y + threadIdx.y;
-    z = blockIdx.z;
-    return x < g.nx && y < g.ny;
+    z = (int)blockIdx.z + a.zlo;
+    return x < a.g.nx && y < a.g.ny;
 }
 
 // Stream-collide of the fluid cell (x, y, z) with the stress stencil read from global memory.
@@ -291,39 +312,46 @@ __device__ __forceinline__ void lb_cell_at(const KArgs<S> &a, int x, int y, int 
 }
 
 // FENE: the stress arrays hold FENE-P conformation tensors (see polymer_force_core_fene)
-template <class S, int PAR, bool FENE = false>
+template <class S, int PAR, bool FENE, bool LIN>
 __global__ void __launch_bounds__(128, lb_min_blocks<S, PAR>()) k_lb(KArgs<S> a) {
     int x, y, z;
-    if (!cell_of_thread(a.g, x, y, z)) return;
-    lb_cell_at<S, PAR, FENE>(a, x, y, z + a.zlo);
+    if (!cell_of_thread<S, LIN>(a, x, y, z)) return;
+    lb_cell_at<S, PAR, FENE>(a, x, y, z);
 }
 
-template <class S>
-__global__ void __launch_bounds__(128) k_fv(KArgs<S> a) {
+// Stress update of the cell (x, y, z) with the stencil read from global memory.
+template <class S, bool VAR>
+__device__ __forceinline__ void fv_cell_at(const KArgs<S> &a, int x, int y, int z) {
     using R = typename Store<S>::R;
     constexpr bool SH = Store<S>::shifted;
-    int x, y, z;
-    if (!cell_of_thread(a.g, x, y, z)) return;
     const Cell cl(a.g, x, y, z);
     const unsigned r = cl.self();
-    const size_t np = (size_t)a.g.np;
+    R tr[6], ur[3], out[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) tr[c] = a.tq[c][r];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ur[j] = a.uiq[j][r];
     const uint32_t m = a.mask[r];
-    R out[6];
     if (m & 1u) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) a.tau_out[c * np + r] = R(0);
-        return;
+        for (int c = 0; c < 6; ++c) out[c] = R(0);
+    } else {
+        const GlobalNb<S> nb{a, cl};
+        fv_core<R, SH, VAR>(a.ph, tr, ur, m, nb, out);
     }
-    R tr[6], ur[3];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) tr[c] = a.tau[c * np + r];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) ur[j] = a.u_in[j * np + r];
-    const GlobalNb<R> gn{a.g, a.ph, cl, a.tau, a.u_in, a.flag, a.parts};
-    const NbAdapter<R> nb{gn};
-    fv_core<R, SH, true>(a.ph, tr, ur, m, nb, out);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) a.tau_out[c * np + r] = out[c];
+    for (int c = 0; c < 6; ++c) a.toq[c][r] = out[c];
+}
+
+// Per-cell stress update, for grids whose z-marching columns would not fill the chip (and
+// all FP64 ones).  Bound by latency there (one round of loads, then the arithmetic), so it
+// is split as finely as it goes: one cell per thread, 128-thread blocks, the neighbours'
+// values through L1 (a 32^3 grid: 256 blocks in 7.7 us, where 8 columns took 20.3).
+template <class S, bool VAR, bool LIN>
+__global__ void __launch_bounds__(128, 5) k_fv_cells(KArgs<S> a) {
+    int x, y, z;
+    if (!cell_of_thread<S, LIN>(a, x, y, z)) return;
+    fv_cell_at<S, VAR>(a, x, y, z);
 }
 
 // Neighbour masks of the cells in a box (whole grid: lo = 0, ext = n) from the flags.
@@ -811,7 +839,7 @@ __device__ __forceinline__ void fv_tile(const KArgs<S> &a, FvSmem<typename Store
 }
 
 template <class S, bool VAR, bool ZR = false, bool W16 = false>
-__global__ void __launch_bounds__(FV_X * FV_Y, sizeof(typename Store<S>::R) == 8 ? 2 : LBVE_FV_MIN_BLOCKS) k_fv_tiled(KArgs<S> a, int zchunk) {
+__global__ void __launch_bounds__(FV_X * FV_Y, LBVE_FV_MIN_BLOCKS) k_fv_tiled(KArgs<S> a, int zchunk) {
     using R = typename Store<S>::R;
     extern __shared__ __align__(16) unsigned char fv_smem_raw[];
     using Sm = FvSmem<R, FvTile<FV_X, W16>::HN>;

@@ -80,6 +80,9 @@ struct Launch {
         a.zlo = d.zlo;
         a.zhi = d.zhi > 0 ? d.zhi : d.g.nz;
         a.key_base = d.key_base;
+        a.lin = (unsigned)((long long)d.g.nx * d.g.ny * zcount(d));
+        a.dnx = FastDiv::of((unsigned)d.g.nx);
+        a.dny = FastDiv::of((unsigned)d.g.ny);
         link_dirs<S>(a);
         return a;
     }
@@ -166,34 +169,91 @@ struct Launch {
         return cudaGetLastError();
     }
     static int lb_rows_used(const DevState &d) { return d.auto_kernels && rows_ok(d) ? 1 : 0; }
-    static cudaError_t lb(const DevState &d, int parity, cudaStream_t s) {
-        if (d.auto_kernels && rows_ok(d)) return lb_rows(d, parity, s);
-        KArgs<S> a = args(d);
-        if (d.ph.fene) {  // the polymer force takes the stress of each cell's conformation
-            if (parity == 0)
-                k_lb<S, 0, true><<<grid2(d), block2(d), 0, s>>>(a);
-            else
-                k_lb<S, 1, true><<<grid2(d), block2(d), 0, s>>>(a);
-        } else if (parity == 0) {
-            k_lb<S, 0><<<grid2(d), block2(d), 0, s>>>(a);
-        } else {
-            k_lb<S, 1><<<grid2(d), block2(d), 0, s>>>(a);
-        }
+    // Launch of a per-cell kernel, by x-y tiles or in memory order (see cell_of_thread).  The
+    // order costs a division and a few spilled registers, tiles the lanes beyond the grid:
+    // measured on GB300 (stream-collide, event-timed, FP32, nx x 64 x 64, tiles against
+    // order) 33: 12.3 / 10.3 us, 110: 20.2 / 19.5, 120: 19.4 / 20.8, 240: 42.0 / 43.8; BF16
+    // 165: 26.5 / 25.5.  The line lies at 7/8 of the lanes in use.
+    template <class K>
+    static cudaError_t cell_launch(const DevState &d, K tiled, K linear, cudaStream_t s) {
+        const KArgs<S> a = args(d);
+        const dim3 b = block2(d), g = grid2(d);
+        if (8LL * d.g.nx * d.g.ny >= 7LL * g.x * b.x * g.y * b.y)
+            tiled<<<g, b, 0, s>>>(a);
+        else
+            linear<<<(a.lin + 127u) / 128u, 128, 0, s>>>(a);
         return cudaGetLastError();
     }
-    // z-planes per block of the z-marching stress update (enough blocks for ~16 waves)
+    static cudaError_t lb(const DevState &d, int parity, cudaStream_t s) {
+        if (d.auto_kernels && rows_ok(d)) return lb_rows(d, parity, s);
+        if (d.ph.fene)  // the polymer force takes the stress of each cell's conformation
+            return parity == 0 ? cell_launch(d, k_lb<S, 0, true, false>, k_lb<S, 0, true, true>, s)
+                               : cell_launch(d, k_lb<S, 1, true, false>, k_lb<S, 1, true, true>, s);
+        return parity == 0 ? cell_launch(d, k_lb<S, 0, false, false>, k_lb<S, 0, false, true>, s)
+                           : cell_launch(d, k_lb<S, 1, false, false>, k_lb<S, 1, false, true>, s);
+    }
+    // The per-cell stress kernel (k_fv_cells).  FP64: every grid (its time is the FP64 pipe's,
+    // which every SM has to share in from the first cells on; measured on GB300, event-timed,
+    // tiled against per-cell: 4 x 32 x 4 98.9 / 18.7 us, 32^3 375 / 29.1, 90^3 733 / 433).
+    // Shifted modes: below 3 * 2^18 cells under schedule AUTO (FP32 tiled against
+    // per-cell: 32^3 20.3 / 7.7 us, 64^3 22.5 / 12.6, 83^3 30.3 / 20.8, 100^3 32.4 / 35.3: the
+    // z-marching columns are too few for the chip on small grids, the per-cell kernel's
+    // re-reads through L1 and L2 cost more on large ones).
+    static bool fv_cells_ok(const DevState &d) {
+        if (!Store<S>::shifted) return true;
+        return d.auto_kernels == 1 && d.g.n < 3LL * (1LL << 18);
+    }
+    static cudaError_t fv_cells(const DevState &d, cudaStream_t s) {
+        return fv_variant(d) ? cell_launch(d, k_fv_cells<S, true, false>, k_fv_cells<S, true, true>, s)
+                             : cell_launch(d, k_fv_cells<S, false, false>, k_fv_cells<S, false, true>, s);
+    }
+    static int sm_count() {
+        int dev = 0, sms = 148;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        return sms;
+    }
+    // z-planes per block of the z-marching stress kernels on tiles columns of nz planes with
+    // `resident` blocks on the device: ~16 waves, at least 16 planes (each chunk stages two
+    // halo planes more than it updates) ...
+    static int march_zchunk(long long tiles, int nz, long long resident) {
+        const long long chunks = (16 * resident + tiles - 1) / tiles;
+        long long zc = (nz + chunks - 1) / chunks;
+        if (zc < 16) zc = 16;
+        return (int)std::min<long long>(zc, nz);
+    }
+    // ... of the batched kernel, whose grid all the members share
+    static int fv_zchunk_batched(const DevState &d) {
+        const long long tiles = (long long)((d.g.nx + FV_X - 1) / FV_X) * ((d.g.ny + FV_Y - 1) / FV_Y);
+        return march_zchunk(tiles, zcount(d), LBVE_FV_MIN_BLOCKS * (long long)sm_count());
+    }
+    // ... of the tiled kernel of a single solve.  Grids too small for 16 waves of 16-plane
+    // chunks take the chunk of least predicted time: a block spends about 0.76 us on a plane
+    // when its SM is full and 1.4 us when it is alone (measured on GB300, FP32), over
+    // zc + 2 planes, a full wave at a time and then the rest.  128^3: 9 planes, 48 us (16
+    // planes 53, 4 planes 52); 100^3: 8 planes, 32.4 us (16 planes 39); 192 x 160 x 96 stays
+    // at 16 planes (12 planes 4 % slower).
     static int fv_zchunk(const DevState &d) {
         const int nz = zcount(d);
         if (d.fv_zchunk > 0) return d.fv_zchunk < nz ? d.fv_zchunk : nz;
         const long long tiles = (long long)((d.g.nx + FV_X - 1) / FV_X) * ((d.g.ny + FV_Y - 1) / FV_Y);
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const long long want = 16LL * LBVE_FV_MIN_BLOCKS * sms;  // ~16 waves of resident blocks
-        const long long chunks = (want + tiles - 1) / tiles;
-        long long zc = (nz + chunks - 1) / chunks;
-        if (zc < 16) zc = 16;
-        if (zc > nz) zc = nz;
-        return (int)zc;
+        const long long sms = sm_count(), resident = LBVE_FV_MIN_BLOCKS * sms;
+        int best = march_zchunk(tiles, nz, resident);
+        if (best > 16) return best;
+        auto cost = [&](int zc) -> double {
+            const long long blocks = tiles * ((nz + zc - 1) / zc), rest = (blocks % resident + sms - 1) / sms;
+            const double full = 0.76 * LBVE_FV_MIN_BLOCKS * (double)(blocks / resident);
+            return (zc + 2) * (full + (rest > 0 ? std::max(1.4, 0.76 * (double)rest) : 0.0));
+        };
+        double c = cost(best);
+        for (int zc : {14, 12, 10, 9, 8, 6, 4}) {
+            if (zc >= nz) continue;
+            const double cz = cost(zc);
+            if (cz < c) {
+                c = cz;
+                best = zc;
+            }
+        }
+        return best;
     }
     // the VAR builds of the stress kernels: a finite-volume variant, FENE-P, or the flux or
     // the source switched off (the plain build has both on at compile time)
@@ -210,11 +270,11 @@ struct Launch {
         k_fv_tiled<S, VAR, ZR, W16><<<nblk, FV_X * FV_Y, sm, s>>>(a, zc);
         return cudaGetLastError();
     }
-    // planes staged by 16-byte copies: 4-byte reals, rows of whole 16-byte chunks and
-    // 16-byte aligned stress and velocity arrays
+    // planes staged by 16-byte copies: rows of whole 16-byte chunks and 16-byte aligned
+    // stress and velocity arrays
     static bool fv_w16(const DevState &d) {
         auto al = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
-        return sizeof(R) == 4 && d.g.nx % 4 == 0 && al(d.tau[0]) && al(d.tau[1]) && al(d.u[0]) && al(d.u[1]);
+        return d.g.nx % 4 == 0 && al(d.tau[0]) && al(d.tau[1]) && al(d.u[0]) && al(d.u[1]);
     }
     template <bool VAR>
     static cudaError_t fv_var(const DevState &d, cudaStream_t s) {
@@ -222,9 +282,7 @@ struct Launch {
         const int tiles = ((d.g.nx + FV_X - 1) / FV_X) * ((d.g.ny + FV_Y - 1) / FV_Y);
         const unsigned nblk = (unsigned)(tiles * ((zcount(d) + zc - 1) / zc));
         const bool zr = d.zhi > 0;  // a z-slab: planes [zlo, zhi) only
-        if constexpr (sizeof(R) == 4) {
-            if (fv_w16(d)) return zr ? fv_launch<VAR, true, true>(d, nblk, zc, s) : fv_launch<VAR, false, true>(d, nblk, zc, s);
-        }
+        if (fv_w16(d)) return zr ? fv_launch<VAR, true, true>(d, nblk, zc, s) : fv_launch<VAR, false, true>(d, nblk, zc, s);
         return zr ? fv_launch<VAR, true, false>(d, nblk, zc, s) : fv_launch<VAR, false, false>(d, nblk, zc, s);
     }
     // The two-cell stress kernel (k_fv_pair): schedule AUTO, the shifted modes' plain
@@ -248,14 +306,7 @@ struct Launch {
         const int nz = zcount(d);
         if (d.fv_zchunk > 0) return d.fv_zchunk < nz ? d.fv_zchunk : nz;
         const long long tiles = (long long)((d.g.nx + FP_TX - 1) / FP_TX) * ((d.g.ny + FP_TY - 1) / FP_TY);
-        int dev = 0, sms = 148;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const long long want = 16LL * 2 * sms;
-        const long long chunks = (want + tiles - 1) / tiles;
-        long long zc = (nz + chunks - 1) / chunks;
-        if (zc < 16) zc = 16;
-        if (zc > nz) zc = nz;
-        return (int)zc;
+        return march_zchunk(tiles, nz, 2LL * sm_count());
     }
     static cudaError_t fv_pair(const DevState &d, cudaStream_t s) {
         if constexpr (!Store<S>::shifted) {
@@ -278,8 +329,10 @@ struct Launch {
         }
     }
     static cudaError_t fv(const DevState &d, cudaStream_t s) {
+        if (fv_cells_ok(d)) return fv_cells(d, s);
         if (fv_pair_ok(d)) return fv_pair(d, s);
-        return fv_variant(d) ? fv_var<true>(d, s) : fv_var<false>(d, s);
+        if constexpr (Store<S>::shifted) return fv_variant(d) ? fv_var<true>(d, s) : fv_var<false>(d, s);
+        return cudaErrorInvalidValue;  // FP64 took the per-cell kernel
     }
     static cudaError_t momentum_exchange(const DevState &d, int parity, const long long *links, const int *seg_begin,
                                          const int *seg_count, int nseg, int max_len, double *contrib, cudaStream_t s) {
@@ -437,7 +490,7 @@ struct Launch {
         e.lb_first = lb_first;
         e.lb_items = ((d.g.nx + e.lb_tx - 1) / e.lb_tx) * ((d.g.ny + lth - 1) / lth) * d.g.nz;
         e.fv_first = fv_first;
-        e.fv_zchunk = fv_zchunk > 0 ? fv_zchunk : fv_zchunk_of(d);
+        e.fv_zchunk = fv_zchunk > 0 ? fv_zchunk : fv_zchunk_batched(d);
         e.fv_items = ((d.g.nx + e.fv_tx - 1) / e.fv_tx) * ((d.g.ny + fth - 1) / fth) *
                      ((d.g.nz + e.fv_zchunk - 1) / e.fv_zchunk);
         *lb_items = e.lb_items;
