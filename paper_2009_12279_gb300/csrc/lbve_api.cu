@@ -376,6 +376,30 @@ void prefault_output(void *p, size_t bytes) {
 // Advance a pool's device step counter (after each step's stream-collide).
 __global__ void k_step_count(unsigned *dstep) { *dstep += 1u; }
 
+PartScratch part_scratch(const lbve_ctx *c) {
+    PartScratch ps;
+    ps.nparts = c->nparts;
+    ps.first_seg = (int)c->wall_seg_begin.size();
+    ps.kind = c->pkind;
+    ps.nf = c->pnf;
+    ps.delta = c->pdelta;
+    ps.diag = c->pdiag;
+    ps.conv = c->pconv;
+    ps.links = c->links;
+    ps.seg_begin = c->seg_begin;
+    ps.seg_count = c->seg_count;
+    ps.capacity = c->part_cap;
+    ps.nbody = c->nbody;
+    ps.max_seg_len = c->max_seg_len;
+    ps.seg_flag = c->seg_flag;
+    ps.contrib = c->contrib;
+    ps.body_F = c->body_F;
+    return ps;
+}
+
+// True when the particle phase of a step sums the step's momentum exchange itself.
+bool phase_sums(const lbve_ctx *c) { return c->nparts > 0 && c->p.pdf_prec != LBVE_F64; }
+
 // Launch the per-body force / torque sums of a context's momentum exchange.
 cudaError_t body_sums(const lbve_ctx *c, PartDev *parts, cudaStream_t st) {
     if (c->p.pdf_prec == LBVE_F64)
@@ -1085,7 +1109,7 @@ lbve_status lbve_step(lbve_ctx *c, int nsteps) {
             CK(c->kt->momentum_exchange(c->d, parity, c->links, c->seg_begin, c->seg_count, c->nbody, c->max_seg_len,
                                         c->contrib, c->stream),
                "momentum exchange");
-            CK(body_sums(c, c->d.parts, c->stream), "body sums");
+            if (!phase_sums(c)) CK(body_sums(c, c->d.parts, c->stream), "body sums");
             CK(timed_end(c), "timing");
         }
         CK(timed_begin(c, LBVE_KT_LB), "timing");
@@ -1098,12 +1122,7 @@ lbve_status lbve_step(lbve_ctx *c, int nsteps) {
         c->d.cur ^= 1;
         if (c->nparts > 0) {
             CK(timed_begin(c, LBVE_KT_PARTICLE), "timing");
-            CK(c->kt->particle_update(c->d, c->nparts, c->stream), "particle update");
-            CK(c->kt->fill_drain(c->d, parity ^ 1, c->nparts, c->pkind, c->pnf, c->pdelta, c->pconv, c->pdiag, c->stream),
-               "fill/drain");
-            CK(c->kt->particle_links(c->d, c->nparts, c->links, c->seg_begin, c->seg_count,
-                                     (int)c->wall_seg_begin.size(), c->part_cap, c->stream),
-               "particle links");
+            CK(c->kt->particle_phase(c->d, parity ^ 1, part_scratch(c), c->stream), "particle phase");
             CK(timed_end(c), "timing");
         }
         c->t++;
@@ -1557,18 +1576,7 @@ lbve_status build_entries(lbve_pool *P) {
     for (lbve_ctx *c : P->members) {
         if (c->nparts <= 0) continue;
         phost.resize(pb * (size_t)(np_ + 1));
-        PartScratch ps;
-        ps.nparts = c->nparts;
-        ps.first_seg = (int)c->wall_seg_begin.size();
-        ps.kind = c->pkind;
-        ps.nf = c->pnf;
-        ps.delta = c->pdelta;
-        ps.diag = c->pdiag;
-        ps.conv = c->pconv;
-        ps.links = c->links;
-        ps.seg_begin = c->seg_begin;
-        ps.seg_count = c->seg_count;
-        ps.capacity = c->part_cap;
+        const PartScratch ps = part_scratch(c);
         P->kt->fill_part_entry(c->d, (int)((c->t + 1) & 1), ps, phost.data() + pb * (size_t)np_);
         ++np_;
     }
@@ -1643,7 +1651,7 @@ lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
             PCK(c->kt->momentum_exchange(d, parity, c->links, c->seg_begin, c->seg_count, c->nbody, c->max_seg_len,
                                          c->contrib, st),
                 "pool momentum exchange");
-            PCK(body_sums(c, d.parts, st), "pool body sums");
+            if (!phase_sums(c)) PCK(body_sums(c, d.parts, st), "pool body sums");
             return LBVE_OK;
         });
         if (s != LBVE_OK) return s;

@@ -63,6 +63,11 @@ struct PartScratch {
     const int *seg_begin;
     int *seg_count;
     const int *capacity;
+    // bodies (wall classes and particles) and their momentum-exchange contributions
+    int nbody, max_seg_len;
+    const int *seg_flag;
+    const double *contrib;
+    double *body_F;
 };
 
 // Device buffers of one solve.
@@ -111,11 +116,12 @@ struct KernelTable {
     cudaError_t (*momentum_exchange)(const DevState &, int parity, const long long *links, const int *seg_begin,
                                      const int *seg_count, int nseg, int max_len, double *contrib, cudaStream_t);
     cudaError_t (*voxelise)(const DevState &, int p, const PartDev &host, cudaStream_t);
-    cudaError_t (*particle_update)(const DevState &, int nparts, cudaStream_t);
     cudaError_t (*particle_links)(const DevState &, int nparts, long long *links, const int *seg_begin, int *seg_count,
                                   int first_seg, const int *capacity, cudaStream_t);
-    cudaError_t (*fill_drain)(const DevState &, int parity, int nparts, uint8_t *kind, uint8_t *nf, double *delta,
-                              int *conv, double *diag, cudaStream_t);
+    // particle phase of one solve after its stress update: in the reduced modes the body
+    // sums of the step's momentum exchange, then the particles' update, fill/drain (on PDFs
+    // in AA parity `parity`) and links
+    cudaError_t (*particle_phase)(const DevState &, int parity, const PartScratch &, cudaStream_t);
     cudaError_t (*read)(const DevState &, int parity, double *rho, double *u, double *tau, int z0, int z1,
                         long long ld, cudaStream_t);
     cudaError_t (*pdfs_io)(const DevState &, int parity, double *io, int write, cudaStream_t);
@@ -140,8 +146,8 @@ struct KernelTable {
     void (*batch_tiles)(const DevState &, int lb_tx, int fv_tx, int *lb_eff, int *fv_eff);
     int (*fv_zchunk_of)(const DevState &);  // z-planes per block the stress kernel will use
     int (*fv_variant_of)(const DevState &);  // 1 when the solve uses a finite-volume variant
-    // pools: the particle phase (update, fill/drain, links) of every member with
-    // particles in one launch; entries built per member like the batch entries
+    // pools: the particle phase of every member with particles in one launch; entries
+    // built per member like the batch entries
     size_t part_entry_bytes;
     void (*fill_part_entry)(const DevState &, int parity0, const PartScratch &, void *entry);
     cudaError_t (*particle_phase_batched)(const void *entries, int n, int k, cudaStream_t);

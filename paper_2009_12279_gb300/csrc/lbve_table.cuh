@@ -6,6 +6,7 @@
 #include <atomic>
 
 #include "lbve_kernels.cuh"
+#include "lbve_particles.cuh"
 #include "lbve_rows.cuh"
 
 namespace lbve {
@@ -375,27 +376,11 @@ struct Launch {
         const BBox b = particle_bbox(d.g, host.X, host.R, 3);
         return build_mask(d, b.lo[0], b.lo[1], b.lo[2], b.ext[0], b.ext[1], b.ext[2], s);
     }
-    static cudaError_t particle_update(const DevState &d, int nparts, cudaStream_t s) {
-        if (nparts <= 0) return cudaSuccess;
-        k_particle_update<S><<<1, 64, 0, s>>>(d.parts, nparts);
-        return cudaGetLastError();
-    }
     static cudaError_t particle_links(const DevState &d, int nparts, long long *links, const int *seg_begin,
                                       int *seg_count, int first_seg, const int *capacity, cudaStream_t s) {
         if (nparts <= 0) return cudaSuccess;
-        k_particle_links<S><<<nparts, 256, 0, s>>>(d.g, d.parts, d.flag, links, seg_begin, seg_count, first_seg,
-                                                   capacity);
-        return cudaGetLastError();
-    }
-    static cudaError_t fill_drain(const DevState &d, int parity, int nparts, uint8_t *kind, uint8_t *nf, double *delta,
-                                  int *conv, double *diag, cudaStream_t s) {
-        if (nparts <= 0) return cudaSuccess;
-        KArgs<S> a = args(d);
-        R *tau = (R *)d.tau[d.cur];
-        if (parity == 0)
-            k_fill_drain<S, 0><<<1, 512, 0, s>>>(a, d.parts, nparts, d.flag, d.mask, tau, kind, nf, delta, conv, diag);
-        else
-            k_fill_drain<S, 1><<<1, 512, 0, s>>>(a, d.parts, nparts, d.flag, d.mask, tau, kind, nf, delta, conv, diag);
+        k_particle_links<S><<<nparts * PC, PT, 0, s>>>(d.g, d.parts, d.flag, links, seg_begin, seg_count, first_seg,
+                                                       capacity);
         return cudaGetLastError();
     }
     static cudaError_t build_mask_impl(const DevState &d, int lx, int ly, int lz, int ex, int ey, int ez,
@@ -540,14 +525,7 @@ struct Launch {
         return per;
     }
     static int fv_variant_of(const DevState &d) { return fv_variant(d) ? 1 : 0; }
-    // d: the member's state when the entries are built; step k after that uses the stress
-    // ping-pong after the step's swap (cur ^ 1 for even k) and AA parity parity0 ^ (k & 1)
-    static void fill_part_entry(const DevState &d, int parity0, const PartScratch &ps, void *entry) {
-        PartEntry<S> &e = *reinterpret_cast<PartEntry<S> *>(entry);
-        DevState d0 = d;
-        d0.cur ^= 1;
-        e.a[0] = args(d0);
-        e.a[1] = args(d);
+    static void part_entry(const PartScratch &ps, const DevState &d, int parity0, PartEntry<S> &e) {
         e.parity0 = parity0;
         e.nparts = ps.nparts;
         e.first_seg = ps.first_seg;
@@ -563,10 +541,34 @@ struct Launch {
         e.seg_begin = ps.seg_begin;
         e.seg_count = ps.seg_count;
         e.capacity = ps.capacity;
+        e.sums = Store<S>::shifted ? ps.contrib : nullptr;  // FP64: summed in link order before
+        e.sum_stride = (ps.max_seg_len + 127) / 128;
+        e.nbody = ps.nbody;
+        e.seg_flag = ps.seg_flag;
+        e.body_F = ps.body_F;
+    }
+    // d: the member's state when the entries are built; step k after that uses the stress
+    // ping-pong after the step's swap (cur ^ 1 for even k) and AA parity parity0 ^ (k & 1)
+    static void fill_part_entry(const DevState &d, int parity0, const PartScratch &ps, void *entry) {
+        PartEntry<S> &e = *reinterpret_cast<PartEntry<S> *>(entry);
+        DevState d0 = d;
+        d0.cur ^= 1;
+        e.a[0] = args(d0);
+        e.a[1] = args(d);
+        part_entry(ps, d, parity0, e);
     }
     static cudaError_t particle_phase_batched(const void *entries, int n, int k, cudaStream_t s) {
         if (n <= 0) return cudaSuccess;
-        k_particle_phase_batched<S><<<n, 512, 0, s>>>((const PartEntry<S> *)entries, k);
+        k_particle_phase<S><<<n * PC, PT, 0, s>>>((const PartEntry<S> *)entries, PartEntry<S>{}, k);
+        return cudaGetLastError();
+    }
+    // one solve, d its state after the step's stress update
+    static cudaError_t particle_phase(const DevState &d, int parity, const PartScratch &ps, cudaStream_t s) {
+        if (ps.nparts <= 0) return cudaSuccess;
+        PartEntry<S> e{};
+        e.a[0] = args(d);
+        part_entry(ps, d, parity, e);
+        k_particle_phase<S><<<PC, PT, 0, s>>>(nullptr, e, 0);
         return cudaGetLastError();
     }
     // resident blocks of the persistent grids: which = 0 for the stream-collide, else the
@@ -607,7 +609,7 @@ template <class S>
 const KernelTable *Launch<S>::table(int prec) {
         static const KernelTable t = {prec,           sizeof(S),        sizeof(R),   &init,
                                       &lb,            &fv,              &momentum_exchange, &voxelise,
-                                      &particle_update, &particle_links, &fill_drain, &read,
+                                      &particle_links, &particle_phase, &read,
                                       &pdfs_io,       &reduce,          &probe,      &build_mask,
                                       &fused,         sizeof(BatchEntry<S>), &fill_entry, &lb_batched,
                                       &fv_batched,    &batched_grid,    &residual,   &batch_tiles,
