@@ -217,7 +217,9 @@ __device__ __forceinline__ double min_image_1d(double d, int n) {
     return d - (double)n * floor(d / (double)n + 0.5);
 }
 
-// Boundary velocity u_b of the solid cell (xq, yq, zq) with flag fl: zero for a no-slip
+// Boundary velocity u_b of the solid cell (xq, yq, zq) with flag fl, as the velocity field's
+// solid cells hold it (set where flags, wall classes or particles change, so that the step
+// kernels read it like a fluid neighbour's velocity): zero for a no-slip
 // wall, the class velocity for a moving wall (Eq. (ubb)), v + w x (r_b - X) with the
 // minimum-image lever arm for a particle cell (Eq. (surface-velocity)).
 template <class R>
@@ -243,38 +245,6 @@ __device__ __forceinline__ void boundary_velocity(const Geo &g, const Phys<R> &p
         ub[0] = (R)(P.v[0] + (P.w[1] * d[2] - P.w[2] * d[1]));
         ub[1] = (R)(P.v[1] + (P.w[2] * d[0] - P.w[0] * d[2]));
         ub[2] = (R)(P.v[2] + (P.w[0] * d[1] - P.w[1] * d[0]));
-    }
-}
-
-// Boundary velocity with the common no-slip case inline and the moving-wall / particle
-// cases out of line (they are rare and would otherwise bloat every caller).
-template <class R>
-struct Vec3 {
-    R x, y, z;
-};
-// Out-of-line wall-class / particle branch of boundary_velocity; the result comes back by
-// value so that callers keep their velocity arrays in registers.
-template <class R>
-__device__ __noinline__ Vec3<R> boundary_velocity_slow(const Geo &g, const Phys<R> &ph, const PartDev *parts, int fl,
-                                                       int xq, int yq, int zq) {
-    R t[3];
-    boundary_velocity<R>(g, ph, parts, fl, xq, yq, zq, t);
-    return Vec3<R>{t[0], t[1], t[2]};
-}
-
-// boundary_velocity with the resting no-slip case inline.
-template <class R>
-__device__ __forceinline__ void boundary_velocity_fast(const Geo &g, const Phys<R> &ph, const PartDev *parts, int fl,
-                                                       int xq, int yq, int zq, R ub[3]) {
-    if (fl == FLAG_NOSLIP) {
-        ub[0] = R(0);
-        ub[1] = R(0);
-        ub[2] = R(0);
-    } else {
-        const Vec3<R> v = boundary_velocity_slow<R>(g, ph, parts, fl, xq, yq, zq);
-        ub[0] = v.x;
-        ub[1] = v.y;
-        ub[2] = v.z;
     }
 }
 
@@ -621,25 +591,13 @@ __device__ __forceinline__ float vpos_open(uint32_t m, int l, float v) {
 __device__ __forceinline__ float2 vpos_open(uint2 m, int l, float2 v) {
     return make_float2(vpos_open(m.x, l, v.x), vpos_open(m.y, l, v.y));
 }
-__device__ __forceinline__ bool lane_moving_solid(uint32_t m, int l, int) {
-    return (m & MASK_MOVING) && nb_solid(m, l + 1);
-}
-__device__ __forceinline__ bool lane_moving_solid(uint2 m, int l, int lane) {
-    return lane_moving_solid(lane == 0 ? m.x : m.y, l, 0);
-}
-__device__ __forceinline__ float &lane_ref(float &v, int) { return v; }
-__device__ __forceinline__ float &lane_ref(float2 &v, int lane) { return lane == 0 ? v.x : v.y; }
-__device__ __forceinline__ float lane_val(float v, int) { return v; }
-__device__ __forceinline__ float lane_val(float2 v, int lane) { return lane == 0 ? v.x : v.y; }
-template <class V>
-__host__ __device__ constexpr int lanes_of() {
-    return sizeof(V) / sizeof(float);
-}
+// a face or edge neighbour of the cell (of either cell) may move
+__device__ __forceinline__ bool any_moving(uint32_t m) { return m & MASK_MOVING; }
+__device__ __forceinline__ bool any_moving(uint2 m) { return (m.x | m.y) & MASK_MOVING; }
 
 // Finite-volume stress update of the shifted modes in lane form (see fv_core for the
 // method): V = float (one cell) or float2 (two cells), M the mask of the lane's cells.
-// nb.u(l, k), nb.tau(l, c): the face-l neighbours' velocity / stress (V); nb.ub(l, lane,
-// out): the boundary velocity of the solid face-l neighbour of the lane's cell.
+// nb.u(l, k), nb.tau(l, c): the face-l neighbours' velocity / stress (V).
 template <class V, class M, bool VAR, class Nb>
 __device__ __forceinline__ void fv_core_sh(const Phys<float> &ph, const V (&tr)[6], const V (&ur)[3], M mask,
                                            const Nb &nb, V out[6]) {
@@ -649,25 +607,20 @@ __device__ __forceinline__ void fv_core_sh(const Phys<float> &ph, const V (&tr)[
     // every face neighbour's u, a solid face's replaced by the mirror value 2 u_b - u(r)
     // (-u(r) at rest), so that the gradient is half the difference of the mirrored values
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int l = 0; l < 6; ++l)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int l = 2 * k + h;
+        for (int j = 0; j < 3; ++j) un[l][j] = vsel_solid(mask, l + 1, vneg(ur[j]), nb.u(l, j));
+    if (any_moving(mask)) {
 #pragma unroll
-            for (int j = 0; j < 3; ++j) un[l][j] = vsel_solid(mask, l + 1, vneg(ur[j]), nb.u(l, j));
+        for (int l = 0; l < 6; ++l)
 #pragma unroll
-            for (int ln = 0; ln < lanes_of<V>(); ++ln) {
-                if (lane_moving_solid(mask, l, ln)) {
-                    float ub[3];
-                    nb.ub(l, ln, ub);
+            for (int j = 0; j < 3; ++j)
+                un[l][j] = vsel_solid(mask, l + 1, vfma(vbc<V>(2.0f), nb.u(l, j), vneg(ur[j])), un[l][j]);
+    }
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) lane_ref(un[l][j], ln) = __fmaf_rn(2.0f, ub[j], -lane_val(ur[j], ln));
-                }
-            }
-        }
+    for (int k = 0; k < 3; ++k)
 #pragma unroll
         for (int j = 0; j < 3; ++j) G[k][j] = vmul(half, vsub(un[2 * k][j], un[2 * k + 1][j]));
-    }
     V net[6];
     const bool flux = !VAR || ph.flux_on;  // without VAR the flux and the source are on
     if (flux) {
@@ -743,42 +696,23 @@ __device__ __forceinline__ void fv_core_sh(const Phys<float> &ph, const V (&tr)[
 // the donor cell's transverse overlap (1 - |u_a|)(1 - |u_b|); ph.divu_on adds tau div u
 // to the source; ph.gk != 0 adds the Giesekus term -(alpha / eta_p)(tau . tau) to it
 // (with the source on).  With VAR false the method's own update is all that is compiled.
-// nb.u(l, k), nb.tau(l, c): velocity / stress of the face-l neighbour (FP64 reads them
-// for fluid neighbours only; the shifted modes read every face neighbour, a solid cell
-// holding zero stress); nb.ub(l, out): boundary velocity of a solid face-l neighbour.
+// nb.u(l, k), nb.tau(l, c): velocity / stress of the face-l neighbour (a solid cell holds
+// its boundary velocity and zero stress).
 // FP64 mode keeps the face-by-face order of the plain statement; shifted modes gather
 // the outflow as (sum of outgoing face velocities) * tau(r).
-// fv_core's neighbour accessor seen by fv_core_sh with one lane (the lane argument of ub
-// is always 0)
-template <class Nb>
-struct OneLaneNb {
-    const Nb &n;
-    __device__ __forceinline__ float u(int l, int j) const { return n.u(l, j); }
-    __device__ __forceinline__ float tau(int l, int c) const { return n.tau(l, c); }
-    __device__ __forceinline__ void ub(int l, int, float o[3]) const { n.ub(l, o); }
-};
-
 template <class R, bool SH, bool VAR, class Nb>
 __device__ __forceinline__ void fv_core(const Phys<R> &ph, const R (&tr)[6], const R (&ur)[3], uint32_t mask,
                                         const Nb &nb, R out[6]) {
     if constexpr (SH) {
-        fv_core_sh<float, uint32_t, VAR>(ph, tr, ur, mask, OneLaneNb<Nb>{nb}, out);
+        fv_core_sh<float, uint32_t, VAR>(ph, tr, ur, mask, nb, out);
     } else {
         // FP64: the face-by-face order of the plain statement
         R un[6][3];
         R G[3][3];
 #pragma unroll
-        for (int l = 0; l < 6; ++l) {
-            if (!nb_solid(mask, l + 1)) {
+        for (int l = 0; l < 6; ++l)
 #pragma unroll
-                for (int j = 0; j < 3; ++j) un[l][j] = nb.u(l, j);
-            } else if (mask & MASK_MOVING) {
-                nb.ub(l, un[l]);
-            } else {  // a resting no-slip wall
-#pragma unroll
-                for (int j = 0; j < 3; ++j) un[l][j] = R(0);
-            }
-        }
+            for (int j = 0; j < 3; ++j) un[l][j] = nb.u(l, j);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const bool fp_ = !nb_solid(mask, 2 * k + 1), fm_ = !nb_solid(mask, 2 * k + 2);

@@ -104,27 +104,30 @@ __device__ __forceinline__ void load_pdfs(const KArgs<S> &a, const Cell &cl, uns
     }
 }
 
-// 6 w_i rho c_i . u_b of a link into a moving wall or particle cell (out of line: rare).
+// Product rounded by itself (FP64 is compiled without contraction).
+__device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul1(double a, double b) { return a * b; }
+
+// 6 w_i rho c_i . u_b of a link into the solid cell nb, whose velocity entries hold u_b.
 template <class R>
-__device__ __noinline__ R moving_wall_term(const Geo &g, const Phys<R> &ph, const PartDev *parts, int fl, int xq,
-                                           int yq, int zq, int i, R rho) {
-    R ub[3];
-    boundary_velocity<R>(g, ph, parts, fl, xq, yq, zq, ub);
+__device__ __forceinline__ R moving_wall_term(R *const (&u)[3], unsigned nb, int i, R rho) {
     R cub = R(0);
     bool first = true;
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const int c = k == 0 ? cx(i) : (k == 1 ? cy(i) : cz(i));
+        const int c = cdir(i, k);
         if (c != 0) {
+            const R ub = u[k][nb];
             if (first) {
-                cub = c > 0 ? ub[k] : -ub[k];
+                cub = c > 0 ? ub : -ub;
                 first = false;
             } else {
-                cub = c > 0 ? cub + ub[k] : cub - ub[k];
+                cub = c > 0 ? cub + ub : cub - ub;
             }
         }
     }
     const R w = i < 7 ? wgt<R>(1) : wgt<R>(7);
-    return R(6) * w * rho * cub;
+    return mul1(mul1(R(6) * w, rho), cub);
 }
 
 // Store post-collision f*_i with AA addressing; links into solid cells bounce back with
@@ -176,10 +179,7 @@ __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, un
                 Store<S>::store16(PAR == 0 ? a.fq[copp(j)] + r : a.fq[j] + nb, bits);
                 if (!nb_solid(mask, j)) continue;
                 S *dst = PAR == 0 ? a.fq[j] + nb : a.fq[copp(j)] + r;
-                const int fl = moving ? (int)a.flag[nb] : FLAG_NOSLIP;
-                const R X = fl == FLAG_NOSLIP ? R(0)
-                                              : moving_wall_term<R>(a.g, a.ph, a.parts, fl, cl.X(cx(j)), cl.Y(cy(j)),
-                                                                    cl.Z(cz(j)), j, rho);
+                const R X = moving ? moving_wall_term<R>(a.uq, nb, j, rho) : R(0);
                 // a boundary at rest (X exactly zero) bounces the normal store's bits
                 Store<S>::store16(dst, X == R(0) ? bits
                                                  : Store<S>::round2(fs[j] - X, fs[j] - X, sc, pair_bits(h, Q + j)));
@@ -203,12 +203,7 @@ __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, un
         const unsigned nb = cl.idx(cx(i), cy(i), cz(i));
         Store<S>::st(PAR == 0 ? a.fq[copp(i)] + r : a.fq[i] + nb, fs[i], sc);
         if (nb_solid(mask, i)) {
-            R X = R(0);
-            if (moving) {
-                const int fl = a.flag[nb];
-                if (fl != FLAG_NOSLIP)
-                    X = moving_wall_term<R>(a.g, a.ph, a.parts, fl, cl.X(cx(i)), cl.Y(cy(i)), cl.Z(cz(i)), i, rho);
-            }
+            const R X = moving ? moving_wall_term<R>(a.uq, nb, i, rho) : R(0);
             Store<S>::st(PAR == 0 ? a.fq[i] + nb : a.fq[copp(i)] + r, fs[i] - X, sc);
         }
     }
@@ -248,7 +243,7 @@ __device__ __forceinline__ void lb_core(const KArgs<S> &a, const Cell &cl, unsig
     lb_core_f<S, PAR>(a, cl, r, mask, tr, tn, f);
 }
 
-// Velocity / stress / boundary-velocity accessors of the face neighbours in global memory
+// Velocity / stress accessors of the face neighbours in global memory
 // (kernel parameters: per-component bases, one multiply-add per address).
 template <class S>
 struct GlobalNb {
@@ -261,11 +256,6 @@ struct GlobalNb {
     }
     __device__ __forceinline__ R u(int l, int j) const { return a.uiq[j][at(l)]; }
     __device__ __forceinline__ R tau(int l, int c) const { return a.tq[c][at(l)]; }
-    __device__ __forceinline__ void ub(int l, R out[3]) const {
-        const int k = l >> 1, s = (l & 1) ? -1 : 1;
-        const int dx = k == 0 ? s : 0, dy = k == 1 ? s : 0, dz = k == 2 ? s : 0;
-        boundary_velocity_fast<R>(a.g, a.ph, a.parts, a.flag[at(l)], cl.X(dx), cl.Y(dy), cl.Z(dz), out);
-    }
 };
 
 // Cell of a thread of the per-cell kernels: blocks of x-y tiles (blockDim (bx, by), grid
@@ -371,15 +361,31 @@ __device__ __forceinline__ uint32_t cell_mask(const Geo &g, const uint8_t *__res
     return m;
 }
 
-// Neighbour masks of the cells of a box (periodically wrapped); a non-fluid cell's stress
-// is set to zero in both stress buffers, so that every solid cell holds zero stress (the
-// shifted-mode stress update reads its face neighbours' stress without a solid test and
-// selects a zero coefficient for a solid face).
+// What the step kernels read at solid cells: the boundary velocity in the velocity field
+// (both buffers of the fused schedule's ping-pong, u0 and u1), so that bounce-back and the
+// velocity gradient need no flag and no FP64 evaluation per link and face, and zero stress
+// (the stress update multiplies it by the zero coefficient of a solid face).
 template <class S>
-__global__ void k_build_mask(Geo g, const uint8_t *__restrict__ flag, uint32_t *__restrict__ mask, int lx, int ly,
-                             int lz, int ex, int ey, int ez, typename Store<S>::R *__restrict__ tau0,
-                             typename Store<S>::R *__restrict__ tau1) {
+__device__ __forceinline__ void set_solid_velocity(const KArgs<S> &a, int x, int y, int z, unsigned r,
+                                                   typename Store<S>::R *u0, typename Store<S>::R *u1) {
     using R = typename Store<S>::R;
+    R ub[3];
+    boundary_velocity<R>(a.g, a.ph, a.parts, a.flag[r], x, y, z, ub);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        u0[j * (size_t)a.g.np + r] = ub[j];
+        u1[j * (size_t)a.g.np + r] = ub[j];
+    }
+}
+
+// Neighbour masks of the cells of a box (periodically wrapped), and what its solid cells
+// hold: boundary velocity, and zero stress in both stress buffers.
+template <class S>
+__global__ void k_build_mask(KArgs<S> a, uint32_t *__restrict__ mask, int lx, int ly, int lz, int ex, int ey, int ez,
+                             typename Store<S>::R *__restrict__ tau0, typename Store<S>::R *__restrict__ tau1,
+                             typename Store<S>::R *u0, typename Store<S>::R *u1) {
+    using R = typename Store<S>::R;
+    const Geo &g = a.g;
     const long long cells = (long long)ex * ey * ez;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < cells;
          k += (long long)gridDim.x * blockDim.x) {
@@ -388,7 +394,7 @@ __global__ void k_build_mask(Geo g, const uint8_t *__restrict__ flag, uint32_t *
         const int y = ((ly + iy) % g.ny + g.ny) % g.ny;
         const int z = ((lz + iz) % g.nz + g.nz) % g.nz;
         const unsigned r = (unsigned)x + (unsigned)g.nx * ((unsigned)y + (unsigned)g.ny * (unsigned)z);
-        const uint32_t m = cell_mask(g, flag, x, y, z);
+        const uint32_t m = cell_mask(g, a.flag, x, y, z);
         mask[r] = m;
         if (m & 1u) {
 #pragma unroll
@@ -396,6 +402,7 @@ __global__ void k_build_mask(Geo g, const uint8_t *__restrict__ flag, uint32_t *
                 tau0[c * (size_t)g.np + r] = R(0);
                 tau1[c * (size_t)g.np + r] = R(0);
             }
+            set_solid_velocity<S>(a, x, y, z, r, u0, u1);
         }
     }
 }
@@ -472,23 +479,13 @@ template <class S>
 struct SmemNb {
     using R = typename Store<S>::R;
     const FusedSmem<R> &sm;
-    const KArgs<S> &a;
-    int sc, sd, su, c2, xg, yg, zg;
+    int sc, sd, su, c2;
     __device__ __forceinline__ int slot(int l) const { return l == 4 ? su : (l == 5 ? sd : sc); }
     __device__ __forceinline__ int cell(int l) const {
         return l == 0 ? c2 + 1 : l == 1 ? c2 - 1 : l == 2 ? c2 + H2X : l == 3 ? c2 - H2X : c2;
     }
     __device__ __forceinline__ R u(int l, int j) const { return sm.in_u[slot(l)][j][cell(l)]; }
     __device__ __forceinline__ R tau(int l, int c) const { return sm.in_tau[slot(l)][c][cell(l)]; }
-    __device__ __forceinline__ void ub(int l, R o[3]) const {
-        const int k = l >> 1, s = (l & 1) ? -1 : 1;
-        int xq = xg + (k == 0 ? s : 0), yq = yg + (k == 1 ? s : 0), zq = zg + (k == 2 ? s : 0);
-        xq = xq < 0 ? xq + a.g.nx : (xq >= a.g.nx ? xq - a.g.nx : xq);
-        yq = yq < 0 ? yq + a.g.ny : (yq >= a.g.ny ? yq - a.g.ny : yq);
-        zq = zq < 0 ? zq + a.g.nz : (zq >= a.g.nz ? zq - a.g.nz : zq);
-        const int fl = a.flag[(unsigned)xq + (unsigned)a.g.nx * ((unsigned)yq + (unsigned)a.g.ny * (unsigned)zq)];
-        boundary_velocity_fast<R>(a.g, a.ph, a.parts, fl, xq, yq, zq, o);
-    }
 };
 
 template <class S, int PAR>
@@ -594,9 +591,7 @@ __global__ void __launch_bounds__(FT_X * FT_Y, sizeof(typename Store<S>::R) == 8
                     for (int c = 0; c < 6; ++c) tr[c] = sm.in_tau[sc][c][c2];
 #pragma unroll
                     for (int j = 0; j < 3; ++j) ur[j] = sm.in_u[sc][j][c2];
-                    const int xg = side_coord(x0 - 1 + hi, a.g.nx, a.g.per[0]);
-                    const int yg = side_coord(y0 - 1 + hj, a.g.ny, a.g.per[1]);
-                    const SmemNb<S> nb{sm, a, sc, sd, su, c2, xg, yg, zg};
+                    const SmemNb<S> nb{sm, sc, sd, su, c2};
                     fv_core<R, SH, true>(a.ph, tr, ur, m, nb, out);
                 }
 #pragma unroll
@@ -676,23 +671,13 @@ template <class S, int HX, int NH>
 struct FvSmemNb {
     using R = typename Store<S>::R;
     const FvSmem<R, NH> &sm;
-    const KArgs<S> &a;
-    int sc, sd, su, c, xg, yg, zg;
+    int sc, sd, su, c;
     __device__ __forceinline__ int slot(int l) const { return l == 4 ? su : (l == 5 ? sd : sc); }
     __device__ __forceinline__ int cell(int l) const {
         return l == 0 ? c + 1 : l == 1 ? c - 1 : l == 2 ? c + HX : l == 3 ? c - HX : c;
     }
     __device__ __forceinline__ R u(int l, int j) const { return sm.u[slot(l)][j][cell(l)]; }
     __device__ __forceinline__ R tau(int l, int cc) const { return sm.tau[slot(l)][cc][cell(l)]; }
-    __device__ __forceinline__ void ub(int l, R o[3]) const {
-        const int k = l >> 1, s = (l & 1) ? -1 : 1;
-        int xq = xg + (k == 0 ? s : 0), yq = yg + (k == 1 ? s : 0), zq = zg + (k == 2 ? s : 0);
-        xq = xq < 0 ? xq + a.g.nx : (xq >= a.g.nx ? xq - a.g.nx : xq);
-        yq = yq < 0 ? yq + a.g.ny : (yq >= a.g.ny ? yq - a.g.ny : yq);
-        zq = zq < 0 ? zq + a.g.nz : (zq >= a.g.nz ? zq - a.g.nz : zq);
-        const int fl = a.flag[(unsigned)xq + (unsigned)a.g.nx * ((unsigned)yq + (unsigned)a.g.ny * (unsigned)zq)];
-        boundary_velocity_fast<R>(a.g, a.ph, a.parts, fl, xq, yq, zq, o);
-    }
 };
 
 // Stress update of work item `item` (TX x TY tile, z-chunk) of one solve; VAR compiles in
@@ -827,7 +812,7 @@ __device__ __forceinline__ void fv_tile(const KArgs<S> &a, FvSmem<typename Store
                 for (int c = 0; c < 6; ++c) tr[c] = sm.tau[sc][c][kc];
 #pragma unroll
                 for (int j = 0; j < 3; ++j) ur[j] = sm.u[sc][j][kc];
-                const FvSmemNb<S, FVH_X, FVH_N> nb{sm, a, sc, sd, su, kc, x, y, z};
+                const FvSmemNb<S, FVH_X, FVH_N> nb{sm, sc, sd, su, kc};
                 fv_core<R, SH, VAR>(a.ph, tr, ur, m, nb, out);
             }
 #pragma unroll
@@ -945,11 +930,10 @@ __global__ void __launch_bounds__(FP_NT, 2) k_fv_pair(KArgs<S> a, int zchunk) {
 #pragma unroll
                 for (int j = 0; j < 3; ++j) ur[j] = ld2(&sm.u[sc][j][kc]);
                 struct Nb {
-                    const KArgs<S> &a;
                     const FvPairSmem &sm;
                     const float2 (&tr)[6];
                     const float2 (&ur)[3];
-                    int sc, sd, su, kc, x, y, z;
+                    int sc, sd, su, kc;
                     __device__ __forceinline__ float2 val(const float (*pl)[FP_HN], int l, int q, float2 own2,
                                                           const float (*pd)[FP_HN], const float (*pu)[FP_HN]) const {
                         switch (l) {
@@ -967,18 +951,8 @@ __global__ void __launch_bounds__(FP_NT, 2) k_fv_pair(KArgs<S> a, int zchunk) {
                     __device__ __forceinline__ float2 tau(int l, int c) const {
                         return val(sm.tau[sc], l, c, tr[c], sm.tau[sd], sm.tau[su]);
                     }
-                    __device__ __forceinline__ void ub(int l, int ln, float o[3]) const {
-                        const int kk = l >> 1, sg = (l & 1) ? -1 : 1;
-                        int xq = x + ln + (kk == 0 ? sg : 0), yq = y + (kk == 1 ? sg : 0), zq = z + (kk == 2 ? sg : 0);
-                        xq = xq < 0 ? xq + a.g.nx : (xq >= a.g.nx ? xq - a.g.nx : xq);
-                        yq = yq < 0 ? yq + a.g.ny : (yq >= a.g.ny ? yq - a.g.ny : yq);
-                        zq = zq < 0 ? zq + a.g.nz : (zq >= a.g.nz ? zq - a.g.nz : zq);
-                        const int fl = a.flag[(unsigned)xq +
-                                              (unsigned)a.g.nx * ((unsigned)yq + (unsigned)a.g.ny * (unsigned)zq)];
-                        boundary_velocity_fast<float>(a.g, a.ph, a.parts, fl, xq, yq, zq, o);
-                    }
                 };
-                const Nb nb{a, sm, tr, ur, sc, sd, su, kc, x, y, z};
+                const Nb nb{sm, tr, ur, sc, sd, su, kc};
                 fv_core_sh<float2, uint2, false>(a.ph, tr, ur, m, nb, out);
 #pragma unroll
                 for (int c = 0; c < 6; ++c) out[c] = make_float2(fa ? out[c].x : 0.0f, fb ? out[c].y : 0.0f);
@@ -1179,10 +1153,11 @@ __device__ __forceinline__ void me_link(const KArgs<S> &a, long long code, doubl
             ci[2] = cz(k);
         }
     const int xb = cl.X(ci[0]), yb = cl.Y(ci[1]), zb = cl.Z(ci[2]);
-    const long long nb = (long long)xb + (long long)a.g.nx * (yb + (long long)a.g.ny * zb);
+    const unsigned nb = (unsigned)xb + (unsigned)a.g.nx * ((unsigned)yb + (unsigned)a.g.ny * (unsigned)zb);
     const int fl = a.flag[nb];
     R ub[3];
-    boundary_velocity<R>(a.g, a.ph, a.parts, fl, xb, yb, zb, ub);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ub[k] = a.uq[k][nb];
     R cub = R(0);
     {
         bool first = true;

@@ -584,7 +584,8 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
 // Particle phase of one step for one solve per cluster: sums of the momentum-exchange
 // partials (reduced modes), symplectic Euler, fill/drain of the cells the spheres now cover
 // or have left (the particles one after another), links of the particles whose cells
-// converted.  Every cell of a particle's box is classified each step and few convert, so
+// converted, and the boundary velocities of the cells they cover (set_solid_velocity).
+// Every cell of a particle's box is classified each step and few convert, so
 // the bounds are latency and the FP64 pipe: the cluster spreads the classification and the
 // link list over PC x PT threads and as many SMs, FP64 work runs in single threads or in
 // lanes side by side, and the conversions work on a list.  Before, three kernels of one
@@ -690,6 +691,18 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
                 fill_drain<S, 1>(E, a, P, p, w, nconv, s_pm);
         }
         cl.sync();
+    }
+    // the spheres' surface velocities, by the state the next step works with
+    for (int p = 0; p < E.nparts; ++p) {
+        __syncthreads();
+        if (tid == 0) w = box_walk(a.g, particle_bbox(a.g, E.parts[p].X, E.parts[p].R, 3));
+        __syncthreads();
+        for (int q = rank * PT + tid; q < w.cells; q += PC * PT) {
+            int x, y, z;
+            box_cell(a.g, w, q, x, y, z);
+            const unsigned r = cell_index(a.g, x, y, z);
+            if (E.flag[r] == FLAG_PART0 + p) set_solid_velocity<S>(a, x, y, z, r, a.u_out, a.u_out);
+        }
     }
     for (int p = 0; p < E.nparts; ++p)
         if ((changed >> p) & 1ull)

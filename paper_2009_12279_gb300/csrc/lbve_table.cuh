@@ -388,7 +388,8 @@ struct Launch {
         const long long cells = (long long)ex * ey * ez;
         if (cells <= 0) return cudaSuccess;
         const unsigned nb = (unsigned)std::min<long long>((cells + 255) / 256, 65535);
-        k_build_mask<S><<<nb, 256, 0, s>>>(d.g, d.flag, d.mask, lx, ly, lz, ex, ey, ez, (R *)d.tau[0], (R *)d.tau[1]);
+        k_build_mask<S><<<nb, 256, 0, s>>>(args(d), d.mask, lx, ly, lz, ex, ey, ez, (R *)d.tau[0], (R *)d.tau[1],
+                                           (R *)d.u[0], (R *)d.u[1]);
         return cudaGetLastError();
     }
     static cudaError_t fused(const DevState &d, int parity, int zchunk, cudaStream_t s) {
