@@ -2,10 +2,12 @@
 // Boltzmann with Guo forcing and a D2Q5 finite-volume Oldroyd-B stress update (Kuron et
 // al., arXiv:2009.12279, Sec. "Lid-driven cavity", Sec. "Four-roll mill").
 //
-// Two kernels per step: k2_lb (polymer force, moments, collision, push streaming with
-// bounce-back into the second PDF array; writes u) and k2_fv (stress update from tau^t
-// and u^t).  The 2-D cases of the paper are small (194^2, 214^2 cells), so the PDFs use
-// two arrays and plain per-cell kernels.  FP64 storage keeps f_i and evaluates every
+// Two operators per step: polymer force, moments, collision and push streaming with
+// bounce-back into the second PDF array; and the stress update from tau^t and u^t.
+// k2_steps runs both on a tile (u^t of the cells around it computed again), for several
+// steps in one launch when the grid is resident on the device; k2_lb and k2_fv are the two
+// as kernels of their own, for larger grids.  The 2-D cases of the paper are small
+// (194^2, 214^2 cells), so the PDFs use two arrays.  FP64 storage keeps f_i and evaluates every
 // formula in the operation order of its plain statement (this unit is built with FMA
 // contraction off); FP32 storage keeps the deviation f_i - w_i rho0 and forms the TRT
 // non-equilibrium parts before scaling them by rounded constants, as the 3-D kernels do.
@@ -13,10 +15,12 @@
 
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
 #include "../../include/lbve2d.h"
+#include "lbve_gridbar.cuh"
 
 namespace {
 
@@ -55,23 +59,23 @@ struct Args2 {
     const R *force;  // 2n or nullptr
 };
 
-// neighbour index (periodic wrap), -1 outside a closed side
+// neighbour index (periodic wrap; one step), -1 outside a closed side
 template <class R>
-__device__ __forceinline__ long long nb2(const Args2<R> &a, int x, int y, int dx, int dy) {
+__device__ __forceinline__ int nb2(const Args2<R> &a, int x, int y, int dx, int dy) {
     int qx = x + dx, qy = y + dy;
     if (qx < 0 || qx >= a.nx) {
         if (!a.per[0]) return -1;
-        qx = (qx + a.nx) % a.nx;
+        qx = qx < 0 ? a.nx - 1 : 0;
     }
     if (qy < 0 || qy >= a.ny) {
         if (!a.per[1]) return -1;
-        qy = (qy + a.ny) % a.ny;
+        qy = qy < 0 ? a.ny - 1 : 0;
     }
-    return (long long)qx + (long long)a.nx * qy;
+    return qx + a.nx * qy;
 }
 
 template <class R>
-__device__ __forceinline__ bool fluid2(const Args2<R> &a, long long r) { return r >= 0 && a.flag[r] == 0; }
+__device__ __forceinline__ bool fluid2(const Args2<R> &a, int r) { return r >= 0 && a.flag[r] == 0; }
 
 template <class R>
 __device__ __forceinline__ R cvec(int i, R v0, R v1) {
@@ -84,13 +88,13 @@ __device__ __forceinline__ R cvec(int i, R v0, R v1) {
 
 // Polymer force, Eq. (force) on the D2Q5 faces +x, -x, +y, -y.
 template <class R>
-__device__ __forceinline__ void polymer_force2(const Args2<R> &a, int x, int y, long long r, R Fp[2]) {
+__device__ __forceinline__ void polymer_force2(const Args2<R> &a, int x, int y, int r, R Fp[2]) {
     Fp[0] = R(0);
     Fp[1] = R(0);
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
         const int k = l >> 1, s = (l & 1) ? -1 : 1;
-        const long long nb = nb2(a, x, y, k == 0 ? s : 0, k == 1 ? s : 0);
+        const int nb = nb2(a, x, y, k == 0 ? s : 0, k == 1 ? s : 0);
         const bool fl = fluid2(a, nb);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -104,7 +108,7 @@ __device__ __forceinline__ void polymer_force2(const Args2<R> &a, int x, int y, 
 
 // F = (g + F_field) + F^p and the moments of Eq. (macroscopic-velocity).
 template <class R, bool SH>
-__device__ __forceinline__ void macro2(const Args2<R> &a, int x, int y, long long r, const R (&f)[Q2], R F[2], R &rho,
+__device__ __forceinline__ void macro2(const Args2<R> &a, int x, int y, int r, const R (&f)[Q2], R F[2], R &rho,
                                        R &drho, R u[2]) {
     R Fp[2];
     polymer_force2(a, x, y, r, Fp);
@@ -134,20 +138,10 @@ __device__ __forceinline__ void macro2(const Args2<R> &a, int x, int y, long lon
     }
 }
 
+// Collision and push streaming of a fluid cell with its PDFs, force and moments.
 template <class R, bool SH>
-__global__ void __launch_bounds__(128) k2_lb(Args2<R> a) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= a.nx || y >= a.ny) return;
-    const long long r = (long long)x + (long long)a.nx * y;
-    if (a.flag[r] != 0) return;
-    R f[Q2];
-#pragma unroll
-    for (int i = 0; i < Q2; ++i) f[i] = a.f_in[i * a.n + r];
-    R F[2], rho, drho, u[2];
-    macro2<R, SH>(a, x, y, r, f, F, rho, drho, u);
-    a.u_out[r] = u[0];
-    a.u_out[a.n + r] = u[1];
+__device__ __forceinline__ void collide_push2(const Args2<R> &a, int x, int y, int r, const R (&f)[Q2], const R (&F)[2],
+                                              R rho, R drho, const R (&u)[2]) {
     const R wp = a.ph.omega_p, wm = a.ph.omega_m;
     const R usq = u[0] * u[0] + u[1] * u[1];
     const R uF = u[0] * F[0] + u[1] * F[1];
@@ -195,7 +189,7 @@ __global__ void __launch_bounds__(128) k2_lb(Args2<R> a) {
     // push streaming with bounce-back, Eq. (ubb)
 #pragma unroll
     for (int i = 0; i < Q2; ++i) {
-        const long long nb = nb2(a, x, y, c2x(i), c2y(i));
+        const int nb = nb2(a, x, y, c2x(i), c2y(i));
         if (fluid2(a, nb)) {
             a.f_out[i * a.n + nb] = fs[i];
         } else {
@@ -206,33 +200,27 @@ __global__ void __launch_bounds__(128) k2_lb(Args2<R> a) {
     }
 }
 
-// Eqs. (continuity)-(source) on the D2Q5 faces, explicit Euler.
-template <class R, bool SH>
-__global__ void __launch_bounds__(128) k2_fv(Args2<R> a) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= a.nx || y >= a.ny) return;
-    const long long r = (long long)x + (long long)a.nx * y;
-    if (a.flag[r] != 0) {
-        for (int c = 0; c < 3; ++c) a.tau_out[c * a.n + r] = R(0);
-        return;
-    }
+// Eqs. (continuity)-(source) on the D2Q5 faces, explicit Euler, of a fluid cell.  u(l, q, j):
+// component j of u^t at the face-l neighbour (l < 4, in the order +x, -x, +y, -y) or the
+// cell itself (4), whose index is q.
+template <class R, class U>
+__device__ __forceinline__ void stress2(const Args2<R> &a, int x, int y, int r, const U &u) {
     R tr[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) tr[c] = a.tau[c * a.n + r];
     R G[2][2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const long long np_ = nb2(a, x, y, k == 0 ? 1 : 0, k == 1 ? 1 : 0);
-        const long long nm_ = nb2(a, x, y, k == 0 ? -1 : 0, k == 1 ? -1 : 0);
+        const int np_ = nb2(a, x, y, k == 0 ? 1 : 0, k == 1 ? 1 : 0);
+        const int nm_ = nb2(a, x, y, k == 0 ? -1 : 0, k == 1 ? -1 : 0);
         const bool fp_ = fluid2(a, np_), fm_ = fluid2(a, nm_);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const R ur = a.u_in[j * a.n + r];
+            const R ur = u(4, r, j);
             const R ubp = np_ >= 0 ? a.ub[j * a.n + np_] : R(0);
             const R ubm = nm_ >= 0 ? a.ub[j * a.n + nm_] : R(0);
-            const R up = fp_ ? R(0.5) * (ur + a.u_in[j * a.n + np_]) : ubp;
-            const R um = fm_ ? R(0.5) * (ur + a.u_in[j * a.n + nm_]) : ubm;
+            const R up = fp_ ? R(0.5) * (ur + u(2 * k, np_, j)) : ubp;
+            const R um = fm_ ? R(0.5) * (ur + u(2 * k + 1, nm_, j)) : ubm;
             G[k][j] = up - um;
         }
     }
@@ -241,9 +229,9 @@ __global__ void __launch_bounds__(128) k2_fv(Args2<R> a) {
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
             const int k = l >> 1, s = (l & 1) ? -1 : 1;
-            const long long nb = nb2(a, x, y, k == 0 ? s : 0, k == 1 ? s : 0);
+            const int nb = nb2(a, x, y, k == 0 ? s : 0, k == 1 ? s : 0);
             if (!fluid2(a, nb)) continue;
-            const R uk = a.u_in[k * a.n + r], unk = a.u_in[k * a.n + nb];
+            const R uk = u(4, r, k), unk = u(l, nb, k);
             const R vout = s > 0 ? uk : -uk;
             const R vin = s > 0 ? -unk : unk;
 #pragma unroll
@@ -267,6 +255,110 @@ __global__ void __launch_bounds__(128) k2_fv(Args2<R> a) {
             S = p + q + a.ph.ep_l * (G[i][j] + G[j][i]) - a.ph.inv_l * tr[c];
         }
         a.tau_out[c * a.n + r] = tr[c] - net[c] + S;
+    }
+}
+
+template <class R, bool SH>
+__global__ void __launch_bounds__(128) k2_lb(Args2<R> a) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= a.nx || y >= a.ny) return;
+    const int r = x + a.nx * y;
+    R f[Q2];
+#pragma unroll
+    for (int i = 0; i < Q2; ++i) f[i] = a.f_in[i * a.n + r];
+    if (a.flag[r] != 0) return;
+    R F[2], rho, drho, u[2];
+    macro2<R, SH>(a, x, y, r, f, F, rho, drho, u);
+    a.u_out[r] = u[0];
+    a.u_out[a.n + r] = u[1];
+    collide_push2<R, SH>(a, x, y, r, f, F, rho, drho, u);
+}
+
+template <class R>
+__global__ void __launch_bounds__(128) k2_fv(Args2<R> a) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= a.nx || y >= a.ny) return;
+    const int r = x + a.nx * y;
+    if (a.flag[r] != 0) {
+        for (int c = 0; c < 3; ++c) a.tau_out[c * a.n + r] = R(0);
+        return;
+    }
+    stress2<R>(a, x, y, r, [&](int, int q, int j) { return a.u_in[j * a.n + q]; });
+}
+
+// Whole steps on T2X x T2Y tiles, one cell per thread, for grids whose tiles are all
+// resident on the device.  A 2-D step moves 3-5 MB at the paper's sizes, all of it in L2:
+// its time is the latency of a kernel, and with a kernel per operator two of them and two
+// launch gaps (cavity 196^2, FP32: 12.5 us per step; here 6.3).  Further warps of the block
+// compute the moments of the 2 (T2X + T2Y) cells around its tile alongside, so that the
+// stress update finds u^t in shared memory and a step needs one meeting of the blocks only
+// (grid_barrier; a cooperative launch when nsteps > 1).
+constexpr int T2X = 32, T2Y = 4, T2N = T2X * T2Y, T2RING = 2 * (T2X + T2Y);
+constexpr int T2THREADS = T2N + (T2RING + 31) / 32 * 32;
+template <class R, bool SH>
+__global__ void __launch_bounds__(T2THREADS) k2_steps(Args2<R> a, int nsteps, unsigned *bar, unsigned *status) {
+    constexpr int HX = T2X + 2, HN = HX * (T2Y + 2);
+    __shared__ R su[2][HN];
+    const int tid = (int)threadIdx.x;
+    const int x0 = (int)blockIdx.x * T2X, y0 = (int)blockIdx.y * T2Y;
+    const bool own = tid < T2N;
+    // place of the thread's cell in the tile with its ring: own cells, then the rows below
+    // and above, then the columns left and right.  A ragged tile's ring follows its own last
+    // cells.
+    int hx, hy;
+    const int ex = min(T2X, a.nx - x0), ey = min(T2Y, a.ny - y0), k = tid - T2N;
+    bool used = true;
+    if (own) {
+        hx = 1 + tid % T2X;
+        hy = 1 + tid / T2X;
+        used = hx <= ex && hy <= ey;
+    } else if (k < 2 * T2X) {
+        hx = 1 + k % T2X;
+        hy = k < T2X ? 0 : ey + 1;
+        used = hx <= ex;
+    } else {
+        hx = k - 2 * T2X < T2Y ? 0 : ex + 1;
+        hy = 1 + (k - 2 * T2X) % T2Y;
+        used = k < T2RING && hy <= ey;
+    }
+    const int h = hx + HX * hy;
+    int x = x0 + hx - 1, y = y0 + hy - 1;
+    if (x < 0 || x >= a.nx) {
+        used = used && a.per[0];
+        x = x < 0 ? a.nx - 1 : 0;
+    }
+    if (y < 0 || y >= a.ny) {
+        used = used && a.per[1];
+        y = y < 0 ? a.ny - 1 : 0;
+    }
+    const int r = used ? x + a.nx * y : 0;
+    const bool fluid = used && a.flag[r] == 0;
+    for (int s = 0; s < nsteps; ++s) {
+        R f[Q2], F[2] = {R(0), R(0)}, rho = R(0), drho = R(0), u[2] = {R(0), R(0)};
+        if (fluid) {
+#pragma unroll
+            for (int i = 0; i < Q2; ++i) f[i] = a.f_in[i * a.n + r];
+            macro2<R, SH>(a, x, y, r, f, F, rho, drho, u);
+            su[0][h] = u[0];
+            su[1][h] = u[1];
+        }
+        __syncthreads();
+        if (own && fluid) {
+            collide_push2<R, SH>(a, x, y, r, f, F, rho, drho, u);
+            stress2<R>(a, x, y, r, [&](int l, int, int j) {
+                return su[j][l == 0 ? h + 1 : l == 1 ? h - 1 : l == 2 ? h + HX : l == 3 ? h - HX : h];
+            });
+        } else if (own && used) {
+            for (int c = 0; c < 3; ++c) a.tau_out[c * a.n + r] = R(0);
+        }
+        if (s + 1 == nsteps || !lbve::grid_barrier(bar, (unsigned)s, status)) return;
+        const R *ft = a.f_in, *tt = a.tau;
+        a.f_in = a.f_out;
+        a.f_out = const_cast<R *>(ft);
+        a.tau = a.tau_out;
+        a.tau_out = const_cast<R *>(tt);
     }
 }
 
@@ -295,7 +387,7 @@ __global__ void k2_read(Args2<R> a, double *rho_out, double *u_out, double *tau_
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= a.nx || y >= a.ny) return;
-    const long long r = (long long)x + (long long)a.nx * y;
+    const int r = x + a.nx * y;
     R f[Q2];
 #pragma unroll
     for (int i = 0; i < Q2; ++i) f[i] = a.f_in[i * a.n + r];
@@ -322,6 +414,10 @@ struct lbve2d_ctx {
     void *f[2] = {nullptr, nullptr}, *tau[2] = {nullptr, nullptr}, *u = nullptr, *ub = nullptr, *force = nullptr;
     uint8_t *flag = nullptr;
     double *stage = nullptr;  // FP64 staging, 10 n doubles
+    unsigned *bar = nullptr;    // device word of the grid barrier
+    unsigned *stuck = nullptr;  // mapped host word: 2 once a barrier's bounded wait gave up
+    unsigned *stuck_dev = nullptr;
+    int resident = 0;           // tiles the device holds at once
     Phys2<double> ph;
     std::string err;
 };
@@ -386,17 +482,50 @@ Args2<R> args2(const lbve2d_ctx *c) {
     return a;
 }
 
+// A barrier between steps gave up: the fields are those of different steps.
+bool stuck2(const lbve2d_ctx *c) { return c->stuck && *(volatile const unsigned *)c->stuck != 0u; }
+const char *const kStuck = "the blocks of a multi-step launch gave up waiting for one another";
+
 dim3 block2d() { return dim3(64, 2); }
 dim3 grid2d(const lbve2d_ctx *c) { return dim3((unsigned)((c->p.nx + 63) / 64), (unsigned)((c->p.ny + 1) / 2)); }
 
+dim3 tiles2d(const lbve2d_ctx *c) {
+    return dim3((unsigned)((c->p.nx + T2X - 1) / T2X), (unsigned)((c->p.ny + T2Y - 1) / T2Y));
+}
+
+// nsteps steps: one launch when every tile is resident, else two kernels per step.  The
+// line is the device's (912 FP32 tiles on GB300, about 340^2 cells): beyond it the moments
+// computed twice and the blocks' waves cost more than the second launch (FP32 per step, this
+// kernel once per step against the two: 500^2 24.7 / 20.6 us, 1000^2 92 / 57).
 template <class R, bool SH>
-cudaError_t step_impl(lbve2d_ctx *c) {
-    Args2<R> a = args2<R>(c);
-    k2_lb<R, SH><<<grid2d(c), block2d(), 0, c->stream>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k2_fv<R, SH><<<grid2d(c), block2d(), 0, c->stream>>>(a);
-    return cudaGetLastError();
+cudaError_t step_impl(lbve2d_ctx *c, int nsteps) {
+    const dim3 g = tiles2d(c);
+    const bool fits = (long long)g.x * g.y <= c->resident;
+    if (nsteps > 1 && fits && !lbve::capturing(c->stream)) {
+        Args2<R> a = args2<R>(c);
+        cudaError_t e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
+        if (e != cudaSuccess) return e;
+        void *args[] = {&a, &nsteps, &c->bar, &c->stuck_dev};
+        e = cudaLaunchCooperativeKernel((const void *)k2_steps<R, SH>, g, dim3(T2THREADS), args, 0, c->stream);
+        if (e != cudaSuccess) return e;
+        c->cur ^= nsteps & 1;
+        c->t += nsteps;
+        return cudaSuccess;
+    }
+    for (int k = 0; k < nsteps; ++k) {
+        Args2<R> a = args2<R>(c);
+        if (fits) {
+            k2_steps<R, SH><<<g, T2THREADS, 0, c->stream>>>(a, 1, nullptr, nullptr);
+        } else {
+            k2_lb<R, SH><<<grid2d(c), block2d(), 0, c->stream>>>(a);
+            k2_fv<R><<<grid2d(c), block2d(), 0, c->stream>>>(a);
+        }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        c->cur ^= 1;
+        c->t++;
+    }
+    return cudaSuccess;
 }
 
 // host FP64 field (2n) -> device field of the storage real type
@@ -468,6 +597,12 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
     if (e == cudaSuccess) e = cudaMalloc(&c->ub, 2 * n * c->rb);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->flag, n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->stage, 15 * n * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->bar, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->stuck, sizeof(unsigned), cudaHostAllocMapped);
+    if (e == cudaSuccess) {
+        *c->stuck = 0u;
+        e = cudaHostGetDevicePointer((void **)&c->stuck_dev, c->stuck, 0);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->flag, 0, n, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ub, 0, 2 * n * c->rb, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->u, 0, 2 * n * c->rb, c->stream);
@@ -479,6 +614,8 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
         lbve2d_destroy(c);
         return e == cudaErrorMemoryAllocation ? LBVE_ENOMEM : LBVE_ECUDA;
     }
+    c->resident = c->rb == 8 ? lbve::resident_blocks(k2_steps<double, false>, T2THREADS, 0)
+                             : lbve::resident_blocks(k2_steps<float, true>, T2THREADS, 0);
     lbve_status s = lbve2d_init_fields(c, nullptr, nullptr, nullptr);
     if (s != LBVE_OK) {
         g_err2 = c->err;
@@ -492,8 +629,10 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
 lbve_status lbve2d_destroy(lbve2d_ctx *c) {
     if (!c) return LBVE_EINVAL;
     cudaStreamSynchronize(c->stream);
-    for (void *p : {c->f[0], c->f[1], c->tau[0], c->tau[1], c->u, c->ub, c->force, (void *)c->flag, (void *)c->stage})
+    for (void *p : {c->f[0], c->f[1], c->tau[0], c->tau[1], c->u, c->ub, c->force, (void *)c->flag, (void *)c->stage,
+                    (void *)c->bar})
         if (p) cudaFree(p);
+    if (c->stuck) cudaFreeHost(c->stuck);
     delete c;
     return LBVE_OK;
 }
@@ -554,6 +693,7 @@ lbve_status lbve2d_init_fields(lbve2d_ctx *c, const double *rho, const double *u
     }
     CK2(cudaGetLastError(), "init kernel");
     CK2(cudaStreamSynchronize(c->stream), "init sync");
+    *(volatile unsigned *)c->stuck = 0u;
     c->t = 0;
     return LBVE_OK;
 }
@@ -561,12 +701,8 @@ lbve_status lbve2d_init_fields(lbve2d_ctx *c, const double *rho, const double *u
 lbve_status lbve2d_step(lbve2d_ctx *c, int nsteps) {
     if (!c) return LBVE_EINVAL;
     if (nsteps < 0) return fail2(c, LBVE_EINVAL, "nsteps must be >= 0");
-    for (int k = 0; k < nsteps; ++k) {
-        const cudaError_t e = c->rb == 8 ? step_impl<double, false>(c) : step_impl<float, true>(c);
-        CK2(e, "step kernels");
-        c->cur ^= 1;
-        c->t++;
-    }
+    if (stuck2(c)) return fail2(c, LBVE_ETIMEOUT, kStuck);
+    CK2((c->rb == 8 ? step_impl<double, false>(c, nsteps) : step_impl<float, true>(c, nsteps)), "step kernels");
     return LBVE_OK;
 }
 
@@ -586,6 +722,7 @@ static lbve_status read_impl(lbve2d_ctx *c, double *rho, double *u, double *tau,
     if (tau) CK2(cudaMemcpyAsync(tau, dtau, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, c->stream), "read copy");
     if (f) CK2(cudaMemcpyAsync(f, df, sizeof(double) * 9 * n, cudaMemcpyDeviceToHost, c->stream), "read copy");
     CK2(cudaStreamSynchronize(c->stream), "read sync");
+    if (stuck2(c)) return fail2(c, LBVE_ETIMEOUT, kStuck);
     return LBVE_OK;
 }
 

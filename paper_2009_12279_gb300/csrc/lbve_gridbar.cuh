@@ -1,0 +1,72 @@
+// lbve_gridbar.cuh -- barrier over the blocks of one cooperative launch, with a bounded wait,
+// and the host side of such launches.  For kernels that take several time steps of a grid
+// small enough to be resident on the device as a whole: between steps the blocks meet here
+// instead of at a kernel boundary.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace lbve {
+
+constexpr unsigned long long GB_WAIT_NS = 1000000000ull;  // 1 s
+
+// Barrier number k (0, 1, ...) of the launch on a word that was 0 at its start: the blocks
+// count up to (k + 1) blocks.  False (in every thread of the block) when the wait gave up,
+// after writing 2 to *status; the caller returns then.  The block barriers around the
+// release add and the acquire load make every thread's earlier writes visible to every
+// thread's later reads (PTX causality order); fences of their own would only add to it.
+__device__ __forceinline__ bool grid_barrier(unsigned *word, unsigned k, unsigned *status) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        const unsigned blocks = gridDim.x * gridDim.y * gridDim.z, target = (k + 1u) * blocks;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
+        unsigned long long t0 = 0;
+        ok = 1;
+        for (unsigned n = 0;; ++n) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+            if (v >= target) break;
+            if ((n & 255u) == 255u) {
+                unsigned long long t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0)
+                    t0 = t;
+                else if (t - t0 > GB_WAIT_NS) {
+                    if (status) *(volatile unsigned *)status = 2u;
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+// Blocks of `kernel` that the current device holds at once (0: no cooperative launches).
+template <class K>
+inline int resident_blocks(K kernel, int threads, size_t smem) {
+    int dev = 0, sms = 0, per = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return sms * per;
+}
+
+// True when the stream is being captured (or its state cannot be asked for): the plain
+// launches are recorded then.
+inline bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+} // namespace lbve
