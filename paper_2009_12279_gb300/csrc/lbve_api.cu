@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "../../include/lbve.h"
+#include "lbve_gridbar.cuh"
 #include "lbve_host.h"
 #include "lbve_launch.h"
 
@@ -281,6 +282,8 @@ namespace {
 __global__ void k_body_reduce(const double *__restrict__ contrib, const int *__restrict__ seg_begin,
                               const int *__restrict__ seg_count, const int *__restrict__ seg_flag, int nbody,
                               double *__restrict__ body_F, PartDev *__restrict__ parts) {
+    step_wait();
+    step_next();
     const int b = blockIdx.x;
     if (b >= nbody) return;
     const int beg = seg_begin[b], end = seg_begin[b] + seg_count[b];
@@ -317,6 +320,8 @@ __global__ void __launch_bounds__(192) k_body_partials(const double *__restrict_
                                                        const int *__restrict__ seg_count,
                                                        const int *__restrict__ seg_flag, int nbody,
                                                        double *__restrict__ body_F, PartDev *__restrict__ parts) {
+    step_wait();
+    step_next();
     const int b = blockIdx.x;
     if (b >= nbody) return;
     const int n = (seg_count[b] + 127) / 128;
@@ -401,14 +406,12 @@ PartScratch part_scratch(const lbve_ctx *c) {
 bool phase_sums(const lbve_ctx *c) { return c->nparts > 0 && c->p.pdf_prec != LBVE_F64; }
 
 // Launch the per-body force / torque sums of a context's momentum exchange.
-cudaError_t body_sums(const lbve_ctx *c, PartDev *parts, cudaStream_t st) {
+cudaError_t body_sums(const lbve_ctx *c, PartDev *parts, cudaStream_t st, int pdl = 0) {
     if (c->p.pdf_prec == LBVE_F64)
-        k_body_reduce<<<c->nbody, 1, 0, st>>>(c->contrib, c->seg_begin, c->seg_count, c->seg_flag, c->nbody,
-                                              c->body_F, parts);
-    else
-        k_body_partials<<<c->nbody, 192, 0, st>>>(c->contrib, (c->max_seg_len + 127) / 128, c->seg_count,
-                                                  c->seg_flag, c->nbody, c->body_F, parts);
-    return cudaGetLastError();
+        return launch_step(pdl, k_body_reduce, dim3(c->nbody), dim3(1), 0, st, c->contrib, c->seg_begin, c->seg_count,
+                           c->seg_flag, c->nbody, c->body_F, parts);
+    return launch_step(pdl, k_body_partials, dim3(c->nbody), dim3(192), 0, st, c->contrib, (c->max_seg_len + 127) / 128,
+                       c->seg_count, c->seg_flag, c->nbody, c->body_F, parts);
 }
 
 __global__ void k_final_sum(const double *__restrict__ partial, long long nblocks, double *__restrict__ out) {
@@ -1070,12 +1073,21 @@ bool use_fused(const lbve_ctx *c, int nsteps) {
     return nsteps >= 2;
 }
 
+// While a call enqueues the kernels of a single solve on its stream they are launched as
+// programmatic dependents of one another (on a captured stream as plain launches).
+struct StepLaunches {
+    lbve_ctx *c;
+    explicit StepLaunches(lbve_ctx *ctx) : c(ctx) { c->d.pdl = capturing(c->stream) ? 0 : 1; }
+    ~StepLaunches() { c->d.pdl = 0; }
+};
+
 lbve_status lbve_step(lbve_ctx *c, int nsteps) {
     if (!c) return LBVE_EINVAL;
     if (nsteps < 0) return fail(c, LBVE_EINVAL, "nsteps must be >= 0");
     if (c->pool) return fail(c, LBVE_ESTATE, "a pool member advances through lbve_pool_step");
     if (c->phase_pending) return fail(c, LBVE_ESTATE, "a stream-collide of lbve_step_phase awaits its stress update");
     if (unstable(c)) return fail(c, flag_status(c), unstable_message(c));
+    StepLaunches chain(c);
     if (use_fused(c, nsteps)) {
         // stream-collide of the first step, fused (stress of step t-1 + stream-collide of
         // step t) for the others, stress update of the last step
@@ -1109,7 +1121,7 @@ lbve_status lbve_step(lbve_ctx *c, int nsteps) {
             CK(c->kt->momentum_exchange(c->d, parity, c->links, c->seg_begin, c->seg_count, c->nbody, c->max_seg_len,
                                         c->contrib, c->stream),
                "momentum exchange");
-            if (!phase_sums(c)) CK(body_sums(c, c->d.parts, c->stream), "body sums");
+            if (!phase_sums(c)) CK(body_sums(c, c->d.parts, c->stream, c->d.pdl), "body sums");
             CK(timed_end(c), "timing");
         }
         CK(timed_begin(c, LBVE_KT_LB), "timing");
@@ -1213,6 +1225,7 @@ lbve_status lbve_halo_unpack(lbve_ctx *c, int what, int side, const void *dev_bu
 
 lbve_status lbve_read_fields_device(lbve_ctx *c, double *rho, double *u, double *tau) {
     if (!c) return LBVE_EINVAL;
+    StepLaunches chain(c);
     CK(c->kt->read(c->d, (int)(c->t & 1), rho, u, tau, 0, c->p.nz, c->d.g.n, c->stream), "read kernel");
     return LBVE_OK;
 }

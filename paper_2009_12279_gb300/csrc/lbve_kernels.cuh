@@ -293,6 +293,7 @@ __device__ __forceinline__ void lb_cell_at(const KArgs<S> &a, int x, int y, int 
 #pragma unroll
     for (int c = 0; c < 6; ++c) tr[c] = a.tq[c][r];
     const uint32_t m = a.mask[r];
+    step_next();
     if (m & 1u) return;
     auto tn = [&](int l, int c) -> R {
         const int k = l >> 1, s = (l & 1) ? -1 : 1;
@@ -304,6 +305,7 @@ __device__ __forceinline__ void lb_cell_at(const KArgs<S> &a, int x, int y, int 
 // FENE: the stress arrays hold FENE-P conformation tensors (see polymer_force_core_fene)
 template <class S, int PAR, bool FENE, bool LIN>
 __global__ void __launch_bounds__(128, lb_min_blocks<S, PAR>()) k_lb(KArgs<S> a) {
+    step_wait();
     int x, y, z;
     if (!cell_of_thread<S, LIN>(a, x, y, z)) return;
     lb_cell_at<S, PAR, FENE>(a, x, y, z);
@@ -322,6 +324,7 @@ __device__ __forceinline__ void fv_cell_at(const KArgs<S> &a, int x, int y, int 
 #pragma unroll
     for (int j = 0; j < 3; ++j) ur[j] = a.uiq[j][r];
     const uint32_t m = a.mask[r];
+    step_next();
     if (m & 1u) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) out[c] = R(0);
@@ -339,6 +342,7 @@ __device__ __forceinline__ void fv_cell_at(const KArgs<S> &a, int x, int y, int 
 // values through L1 (a 32^3 grid: 256 blocks in 7.7 us, where 8 columns took 20.3).
 template <class S, bool VAR, bool LIN>
 __global__ void __launch_bounds__(128, 5) k_fv_cells(KArgs<S> a) {
+    step_wait();
     int x, y, z;
     if (!cell_of_thread<S, LIN>(a, x, y, z)) return;
     fv_cell_at<S, VAR>(a, x, y, z);
@@ -797,6 +801,7 @@ __device__ __forceinline__ void fv_tile(const KArgs<S> &a, FvSmem<typename Store
             stage(z + 1 + LBVE_FV_AHEAD);
         else
             cp_async_commit();
+        if (z + 1 == z1) step_next();
         asm volatile("cp.async.wait_group %0;\n" ::"n"(LBVE_FV_AHEAD) : "memory");
         __syncthreads();
         if (own) {
@@ -826,6 +831,7 @@ __device__ __forceinline__ void fv_tile(const KArgs<S> &a, FvSmem<typename Store
 template <class S, bool VAR, bool ZR = false, bool W16 = false>
 __global__ void __launch_bounds__(FV_X * FV_Y, LBVE_FV_MIN_BLOCKS) k_fv_tiled(KArgs<S> a, int zchunk) {
     using R = typename Store<S>::R;
+    step_wait();
     extern __shared__ __align__(16) unsigned char fv_smem_raw[];
     using Sm = FvSmem<R, FvTile<FV_X, W16>::HN>;
     Sm &sm = *reinterpret_cast<Sm *>(fv_smem_raw);
@@ -851,6 +857,7 @@ struct FvPairSmem {
 template <class S, bool ZR>
 __global__ void __launch_bounds__(FP_NT, 2) k_fv_pair(KArgs<S> a, int zchunk) {
     static_assert(Store<S>::shifted, "two-cell stress update: FP32 stress");
+    step_wait();
     extern __shared__ __align__(16) unsigned char fp_smem_raw[];
     FvPairSmem &sm = *reinterpret_cast<FvPairSmem *>(fp_smem_raw);
     const int tid = threadIdx.x;
@@ -915,6 +922,7 @@ __global__ void __launch_bounds__(FP_NT, 2) k_fv_pair(KArgs<S> a, int zchunk) {
             stage(z + 1 + LBVE_FV_AHEAD);
         else
             cp_async_commit();
+        if (z + 1 == z1) step_next();
         asm volatile("cp.async.wait_group %0;\n" ::"n"(LBVE_FV_AHEAD) : "memory");
         __syncthreads();
         if (own) {
@@ -1210,6 +1218,7 @@ __global__ void __launch_bounds__(128) k_momentum_exchange(KArgs<S> a, const lon
                                                            const int *__restrict__ seg_begin,
                                                            const int *__restrict__ seg_count,
                                                            double *__restrict__ contrib) {
+    step_wait();
     const int b = blockIdx.y;
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= seg_count[b]) return;
@@ -1225,6 +1234,8 @@ __global__ void __launch_bounds__(128) k_momentum_exchange_part(KArgs<S> a, cons
                                                                 const int *__restrict__ seg_begin,
                                                                 const int *__restrict__ seg_count,
                                                                 double *__restrict__ part) {
+    step_wait();
+    step_next();
     const int b = blockIdx.y;
     const int cnt = seg_count[b];
     if ((int)blockIdx.x * 128 >= cnt) return;  // the whole block is past this body's links
@@ -1298,6 +1309,7 @@ __global__ void k_read(KArgs<S> a, double *__restrict__ rho_out, double *__restr
                        double *__restrict__ tau_out, int z0, long long ld) {
     using R = typename Store<S>::R;
     constexpr bool SH = Store<S>::shifted;
+    step_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= a.g.nx) return;
     const Cell cl(a.g, x, blockIdx.y, blockIdx.z + z0);

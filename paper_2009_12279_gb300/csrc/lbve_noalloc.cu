@@ -10,6 +10,7 @@
 #include <mutex>
 #include <string>
 
+#include "lbve_gridbar.cuh"
 #include "lbve_host.h"
 #include "lbve_launch.h"
 
@@ -126,6 +127,7 @@ lbve_status lbve_step_noalloc(const lbve_params *p, void *f, void *tau_a, void *
     cudaStream_t s = (cudaStream_t)cuda_stream;
     e = kt->build_mask(d, 0, 0, 0, p->nx, p->ny, p->nz, s);
     if (e != cudaSuccess) return fail(LBVE_ECUDA, std::string("mask kernel: ") + cudaGetErrorString(e));
+    d.pdl = capturing(s) ? 0 : 1;
     for (int k = 0; k < nsteps; ++k) {
         const int parity = (int)((t0 + k) & 1);
         d.step = (unsigned)(t0 + k);

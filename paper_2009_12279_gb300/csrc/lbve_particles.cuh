@@ -595,6 +595,8 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
 template <class S>
 __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
     k_particle_phase(const PartEntry<S> *__restrict__ entries, const __grid_constant__ PartEntry<S> one, int k) {
+    step_wait();
+    step_next();  // its few blocks leave the device to the next kernel's anyway
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     const PartEntry<S> &E = entries ? entries[blockIdx.x / PC] : one;
     const KArgs<S> &a = E.a[k & 1];

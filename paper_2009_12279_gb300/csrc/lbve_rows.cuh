@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(LR_MAX_NX + 32, 1) k_lb_rows(KArgs<S> a, RowsW
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    step_wait();
     const unsigned nxu = (unsigned)nx, nxy = (unsigned)nx * (unsigned)ny;
     auto row_of = [&](int y_, int z_) -> unsigned { return nxu * (unsigned)y_ + nxy * (unsigned)z_; };
     auto pdf_s = [&](int s, int i) -> S * { return reinterpret_cast<S *>(lr_smem + L.stage_off(s)) + (size_t)i * nx; };
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(LR_MAX_NX + 32, 1) k_lb_rows(KArgs<S> a, RowsW
             }
             ++issued;
         }
+        step_next();
         // every copy issued lands before the block exits: wait for the last stages' phases
         if (lane == 0) {
             for (int j = max(0, issued - NS); j < issued; ++j) {
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(LR_MAX_NX + 32, 1) k_lb_rows(KArgs<S> a, RowsW
             if (a.bad != nullptr) *(volatile unsigned *)a.bad = 2u;
             return;
         }
+        if (j + 1 == rows) step_next();
         const int y = y0 + j;
         const uint32_t m = mask_s(s)[x];
         if (!(m & 1u)) {

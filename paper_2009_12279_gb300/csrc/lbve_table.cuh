@@ -163,11 +163,7 @@ struct Launch {
         if (e != cudaSuccess) return e;
         const unsigned nblk = (unsigned)(zcount(d) * w.strips);
         const unsigned nthr = (unsigned)(d.g.nx + 32);
-        if (parity == 0)
-            k_lb_rows<S, 0><<<nblk, nthr, sm, s>>>(a, w);
-        else
-            k_lb_rows<S, 1><<<nblk, nthr, sm, s>>>(a, w);
-        return cudaGetLastError();
+        return launch_step(d.pdl, parity == 0 ? k_lb_rows<S, 0> : k_lb_rows<S, 1>, dim3(nblk), dim3(nthr), sm, s, a, w);
     }
     static int lb_rows_used(const DevState &d) { return d.auto_kernels && rows_ok(d) ? 1 : 0; }
     // Launch of a per-cell kernel, by x-y tiles or in memory order (see cell_of_thread).  The
@@ -180,10 +176,8 @@ struct Launch {
         const KArgs<S> a = args(d);
         const dim3 b = block2(d), g = grid2(d);
         if (8LL * d.g.nx * d.g.ny >= 7LL * g.x * b.x * g.y * b.y)
-            tiled<<<g, b, 0, s>>>(a);
-        else
-            linear<<<(a.lin + 127u) / 128u, 128, 0, s>>>(a);
-        return cudaGetLastError();
+            return launch_step(d.pdl, tiled, g, b, 0, s, a);
+        return launch_step(d.pdl, linear, dim3((a.lin + 127u) / 128u), dim3(128), 0, s, a);
     }
     static cudaError_t lb(const DevState &d, int parity, cudaStream_t s) {
         if (d.auto_kernels && rows_ok(d)) return lb_rows(d, parity, s);
@@ -268,8 +262,7 @@ struct Launch {
         static SmemAttrOnce attr;
         cudaError_t e = attr.ensure(k_fv_tiled<S, VAR, ZR, W16>, sm);
         if (e != cudaSuccess) return e;
-        k_fv_tiled<S, VAR, ZR, W16><<<nblk, FV_X * FV_Y, sm, s>>>(a, zc);
-        return cudaGetLastError();
+        return launch_step(d.pdl, k_fv_tiled<S, VAR, ZR, W16>, dim3(nblk), dim3(FV_X * FV_Y), sm, s, a, zc);
     }
     // planes staged by 16-byte copies: rows of whole 16-byte chunks and 16-byte aligned
     // stress and velocity arrays
@@ -322,11 +315,7 @@ struct Launch {
             const bool zr = d.zhi > 0;  // a z-slab: planes [zlo, zhi) only
             cudaError_t e = zr ? attr[1].ensure(k_fv_pair<S, true>, sm) : attr[0].ensure(k_fv_pair<S, false>, sm);
             if (e != cudaSuccess) return e;
-            if (zr)
-                k_fv_pair<S, true><<<nblk, FP_NT, sm, s>>>(a, zc);
-            else
-                k_fv_pair<S, false><<<nblk, FP_NT, sm, s>>>(a, zc);
-            return cudaGetLastError();
+            return launch_step(d.pdl, zr ? k_fv_pair<S, true> : k_fv_pair<S, false>, dim3(nblk), dim3(FP_NT), sm, s, a, zc);
         }
     }
     static cudaError_t fv(const DevState &d, cudaStream_t s) {
@@ -342,18 +331,13 @@ struct Launch {
         const dim3 g((unsigned)((max_len + 127) / 128), (unsigned)nseg);
         if constexpr (Store<S>::shifted) {
             // reduced modes: per-block partials (nseg x ceil(max_len / 128) of them)
-            if (parity == 0)
-                k_momentum_exchange_part<S, 0><<<g, 128, 0, s>>>(a, links, seg_begin, seg_count, contrib);
-            else
-                k_momentum_exchange_part<S, 1><<<g, 128, 0, s>>>(a, links, seg_begin, seg_count, contrib);
+            return launch_step(d.pdl, parity == 0 ? k_momentum_exchange_part<S, 0> : k_momentum_exchange_part<S, 1>, g,
+                               dim3(128), 0, s, a, links, seg_begin, seg_count, contrib);
         } else {
             // FP64 parity mode: one contribution per link, summed in link order
-            if (parity == 0)
-                k_momentum_exchange<S, 0><<<g, 128, 0, s>>>(a, links, seg_begin, seg_count, contrib);
-            else
-                k_momentum_exchange<S, 1><<<g, 128, 0, s>>>(a, links, seg_begin, seg_count, contrib);
+            return launch_step(d.pdl, parity == 0 ? k_momentum_exchange<S, 0> : k_momentum_exchange<S, 1>, g, dim3(128), 0,
+                               s, a, links, seg_begin, seg_count, contrib);
         }
-        return cudaGetLastError();
     }
     static cudaError_t halo_pack(const DevState &d, int what, int side, int parity, void *buf, cudaStream_t s) {
         KArgs<S> a = args(d);
@@ -416,11 +400,8 @@ struct Launch {
         KArgs<S> a = args(d);
         dim3 g = grid3(d);
         g.z = (unsigned)(z1 - z0);
-        if (parity == 0)
-            k_read<S, 0><<<g, d.block_x, 0, s>>>(a, rho, u, tau, z0, ld);
-        else
-            k_read<S, 1><<<g, d.block_x, 0, s>>>(a, rho, u, tau, z0, ld);
-        return cudaGetLastError();
+        return launch_step(d.pdl, parity == 0 ? k_read<S, 0> : k_read<S, 1>, g, dim3(d.block_x), 0, s, a, rho, u, tau, z0,
+                           ld);
     }
     static cudaError_t pdfs_io(const DevState &d, int parity, double *io, int write, cudaStream_t s) {
         KArgs<S> a = args(d);
@@ -569,8 +550,7 @@ struct Launch {
         PartEntry<S> e{};
         e.a[0] = args(d);
         part_entry(ps, d, parity, e);
-        k_particle_phase<S><<<PC, PT, 0, s>>>(nullptr, e, 0);
-        return cudaGetLastError();
+        return launch_step(d.pdl, k_particle_phase<S>, dim3(PC), dim3(PT), 0, s, nullptr, e, 0);
     }
     // resident blocks of the persistent grids: which = 0 for the stream-collide, else the
     // stress kernel of tile width `which`
