@@ -1116,7 +1116,9 @@ lbve_status lbve_step(lbve_ctx *c, int nsteps) {
     for (int s = 0; s < nsteps; ++s) {
         const int parity = (int)(c->t & 1);
         c->d.step = (unsigned)c->t;
-        if (c->nbody > 0) {
+        // forces on wall classes are those of the call's last step (nothing else reads them);
+        // particles move by theirs, every step
+        if (c->nbody > 0 && (c->nparts > 0 || s + 1 == nsteps)) {
             CK(timed_begin(c, LBVE_KT_ME), "timing");
             CK(c->kt->momentum_exchange(c->d, parity, c->links, c->seg_begin, c->seg_count, c->nbody, c->max_seg_len,
                                         c->contrib, c->stream),
@@ -1651,12 +1653,14 @@ lbve_status fan_out(lbve_pool *P, const std::vector<lbve_ctx *> &list, Body &&bo
 lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
     const int n = (int)P->members.size();
     std::vector<lbve_ctx *> with_bodies, with_parts;
-    for (lbve_ctx *c : P->members) {
-        if (c->nbody > 0) with_bodies.push_back(c);
+    for (lbve_ctx *c : P->members)
         if (c->nparts > 0) with_parts.push_back(c);
-    }
     for (int k = 0; k < nsteps; ++k) {
         const int kk = q + k;  // steps since the entries were built (they encode that state)
+        // members with wall classes only: the forces of the call's last step (see lbve_step)
+        with_bodies.clear();
+        for (lbve_ctx *c : P->members)
+            if (c->nbody > 0 && (c->nparts > 0 || k + 1 == nsteps)) with_bodies.push_back(c);
         lbve_status s = fan_out(P, with_bodies, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
             DevState d = c->d;  // the member's state at the start of this call
             if (k & 1) d.cur ^= 1;
