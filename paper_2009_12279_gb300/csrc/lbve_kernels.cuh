@@ -1246,15 +1246,15 @@ __global__ void __launch_bounds__(128) k_momentum_exchange_part(KArgs<S> a, cons
 #pragma unroll
     for (int k = 0; k < 6; ++k) sh[k][threadIdx.x] = o[k];
     __syncthreads();
-    for (int s = 64; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
+    // a warp per component: halves added until one value is left
+    const int lane = (int)threadIdx.x & 31;
+#pragma unroll 1
+    for (int k = (int)threadIdx.x >> 5; k < 6; k += 4) {
+        double v = (sh[k][lane] + sh[k][lane + 64]) + (sh[k][lane + 32] + sh[k][lane + 96]);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + s];
-        __syncthreads();
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+        if (lane == 0) part[((long long)b * gridDim.x + blockIdx.x) * 8 + k] = v;
     }
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) part[((long long)b * gridDim.x + blockIdx.x) * 8 + k] = sh[k][0];
 }
 
 // ---------------------------------------------------------------------------------

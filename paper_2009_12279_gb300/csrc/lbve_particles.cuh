@@ -15,39 +15,35 @@ struct BBox {
     __host__ __device__ long long cells() const { return (long long)ext[0] * ext[1] * ext[2]; }
 };
 
-// Cells within R + margin of the particle centre (whole domain along a periodic side
-// the box would wrap onto itself; clamped to the domain along a closed side).
+// One side of a particle's box: cells within R + margin of the centre coordinate X (the
+// whole side where a periodic one would wrap onto itself; clamped to the domain along a
+// closed one).
+__host__ __device__ inline void bbox_side(int n, int per, double X, double R, int margin, int &lo, int &ext) {
+    lo = (int)floor(X - R) - margin;
+    int hi = (int)ceil(X + R) + margin;
+    if (!per) {
+        lo = lo < 0 ? 0 : lo;
+        hi = hi > n - 1 ? n - 1 : hi;
+    }
+    ext = hi - lo + 1;
+    if (ext > n) {
+        lo = 0;
+        ext = n;
+    }
+    if (ext < 0) ext = 0;
+}
 __host__ __device__ inline BBox particle_bbox(const Geo &g, const double X[3], double R, int margin) {
     BBox b;
     const int nn[3] = {g.nx, g.ny, g.nz};
-    for (int k = 0; k < 3; ++k) {
-        int lo = (int)floor(X[k] - R) - margin;
-        int hi = (int)ceil(X[k] + R) + margin;
-        if (!g.per[k]) {
-            lo = lo < 0 ? 0 : lo;
-            hi = hi > nn[k] - 1 ? nn[k] - 1 : hi;
-        }
-        int ext = hi - lo + 1;
-        if (ext > nn[k]) {
-            lo = 0;
-            ext = nn[k];
-        }
-        if (ext < 0) ext = 0;
-        b.lo[k] = lo;
-        b.ext[k] = ext;
-    }
+    for (int k = 0; k < 3; ++k) bbox_side(nn[k], g.per[k], X[k], R, margin, b.lo[k], b.ext[k]);
     return b;
 }
-
-__host__ __device__ inline int bbox_capacity_side(double R, int margin) { return 2 * (int)ceil(R) + 2 * margin + 3; }
 
 // A particle's box as the phase walks it: the lower corner wrapped into the domain once, so
 // that a cell's coordinate and a cell's place in the box are each one conditional
 // correction away.
 struct BoxWalk {
-    int lo[3], ext[3];
-    FastDiv dx, dy;
-    int cells;
+    int lo[3], ext[3], cells;
 };
 __device__ __forceinline__ BoxWalk box_walk(const Geo &g, const BBox &b) {
     BoxWalk w;
@@ -57,13 +53,11 @@ __device__ __forceinline__ BoxWalk box_walk(const Geo &g, const BBox &b) {
         w.ext[k] = b.ext[k];
     }
     w.cells = (int)b.cells();
-    w.dx = FastDiv::of((unsigned)(b.ext[0] > 0 ? b.ext[0] : 1));
-    w.dy = FastDiv::of((unsigned)(b.ext[1] > 0 ? b.ext[1] : 1));
     return w;
 }
 // coordinates of cell k of the box
 __device__ __forceinline__ void box_cell(const Geo &g, const BoxWalk &w, int k, int &x, int &y, int &z) {
-    const unsigned row = w.dx.div((unsigned)k), pl = w.dy.div(row);
+    const unsigned row = (unsigned)k / (unsigned)w.ext[0], pl = row / (unsigned)w.ext[1];
     x = w.lo[0] + k - (int)row * w.ext[0];
     y = w.lo[1] + (int)row - (int)pl * w.ext[1];
     z = w.lo[2] + (int)pl;
@@ -113,29 +107,44 @@ __device__ __forceinline__ void min_image(const Geo &g, const double X[3], int x
 // roundings and that of R^2, within 2^-18 D^2 of the FP64 value.  Only in that shell (a
 // few cells in ten thousand) does the FP64 test decide.  (Working on the coordinates
 // themselves needs a shell thousands of times wider, and nearly every warp at the surface
-// then ran the FP64 branch: 33 us per step for an R = 8 sphere, now part of 5.)
+// then ran the FP64 branch: 33 us per step for an R = 8 sphere in one block.)
 struct SphereFilter {
     int Xi[3];
     float Xf[3], R2, tol;
+    float deep2;  // squared distance below which every neighbour lies inside, too
 };
-__device__ __forceinline__ SphereFilter sphere_filter(const Geo &g, const PartDev &P) {
-    SphereFilter f;
-    const int nn[3] = {g.nx, g.ny, g.nz};
-    for (int k = 0; k < 3; ++k) {
-        const double c = rint(P.X[k]);
-        f.Xf[k] = (float)(P.X[k] - c);
-        f.Xi[k] = (int)c;
-        if (g.per[k]) f.Xi[k] = ((f.Xi[k] % nn[k]) + nn[k]) % nn[k];
+// The box and (sf != nullptr) the filter of a particle, a side per lane of one warp (FP64
+// latencies side by side): into shared memory.
+__device__ __forceinline__ void prepare_box(const Geo &g, const PartDev &P, int margin, BoxWalk &w, SphereFilter *sf) {
+    const int lane = (int)threadIdx.x & 31;
+    int ext = 1;
+    if (lane < 3) {
+        const int n = lane == 0 ? g.nx : (lane == 1 ? g.ny : g.nz), per = g.per[lane];
+        const double X = P.X[lane];
+        int lo;
+        bbox_side(n, per, X, P.R, margin, lo, ext);
+        w.lo[lane] = ((lo % n) + n) % n;
+        w.ext[lane] = ext;
+        if (sf) {
+            const double c = rint(X);
+            sf->Xf[lane] = (float)(X - c);
+            const int i = (int)c;
+            sf->Xi[lane] = per ? ((i % n) + n) % n : i;
+        }
+    } else if (lane == 3 && sf) {
+        const double D = P.R + 5.0;
+        sf->R2 = (float)(P.R * P.R);
+        sf->tol = (float)(D * D * 0x1p-18);
+        const float deep = fmaxf((float)P.R - 1.5f, 0.0f);
+        sf->deep2 = deep * deep;
     }
-    const double D = P.R + 5.0;
-    f.R2 = (float)(P.R * P.R);
-    f.tol = (float)(D * D * 0x1p-18);
-    return f;
+    const int e1 = __shfl_sync(0xffffffffu, ext, 1), e2 = __shfl_sync(0xffffffffu, ext, 2);
+    if (lane == 0) w.cells = ext * e1 * e2;
 }
 __device__ __forceinline__ bool inside_sphere(const Geo &g, const PartDev &P, const SphereFilter &f, int x, int y,
-                                              int z) {
+                                              int z, float &d2) {
     const int q[3] = {x, y, z}, nn[3] = {g.nx, g.ny, g.nz};
-    float d2 = 0.0f;
+    d2 = 0.0f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         int i = q[k] - f.Xi[k];
@@ -254,15 +263,15 @@ __device__ __forceinline__ void cluster_exchange(cooperative_groups::cluster_gro
 
 // Boundary links of particle p: every (fluid cell r, direction i) with r + c_i covered by
 // it, in cell order then direction order.  The blocks of the cluster take consecutive
-// ranges of the box; counts first, then the links at their places.
-template <class S>
+// ranges of the box; counts first, then the links at their places.  The neighbour masks
+// tell the few cells that have a moving neighbour, so the others cost one load.
 __device__ __forceinline__ void particle_links(cooperative_groups::cluster_group &cl, const Geo &g, const PartDev &P,
-                                               int p, const uint8_t *flag, long long *links, const int *seg_begin,
-                                               int *seg_count, int seg, int cap, ClusterCounts &counts, int &buf,
-                                               int *wsum) {
+                                               int p, const uint8_t *flag, const uint32_t *mask, long long *links,
+                                               const int *seg_begin, int *seg_count, int seg, int cap,
+                                               ClusterCounts &counts, int &buf, int *wsum) {
     __shared__ BoxWalk w;
     __syncthreads();
-    if (threadIdx.x == 0) w = box_walk(g, particle_bbox(g, P.X, P.R, 2));
+    if (threadIdx.x < 32) prepare_box(g, P, 2, w, nullptr);
     __syncthreads();
     const int rank = (int)cl.block_rank();
     const int per = (w.cells + PC - 1) / PC, lo = min(w.cells, per * rank), hi = min(w.cells, lo + per);
@@ -270,22 +279,36 @@ __device__ __forceinline__ void particle_links(cooperative_groups::cluster_group
         int x, y, z;
         box_cell(g, w, k, x, y, z);
         r = cell_index(g, x, y, z);
-        unsigned m = 0;
-        if (flag[r] != FLAG_FLUID) return 0u;
+        const uint32_t m = mask[r];
+        if ((m & 1u) || !(m & MASK_MOVING)) return 0u;
         const Cell c(g, x, y, z);
+        unsigned d = 0;
+        // set bits, six at a time: their flag loads go out together
+#pragma unroll 1
+        for (uint32_t s = m & 0x7fffeu; s;) {
+            int i[6], f[6];
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const bool out = (!g.per[0] && (x + cx(i) < 0 || x + cx(i) >= g.nx)) ||
-                             (!g.per[1] && (y + cy(i) < 0 || y + cy(i) >= g.ny)) ||
-                             (!g.per[2] && (z + cz(i) < 0 || z + cz(i) >= g.nz));
-            if (!out && flag[c.idx(cx(i), cy(i), cz(i))] == FLAG_PART0 + p) m |= 1u << i;
+            for (int n = 0; n < 6; ++n) {
+                i[n] = s ? __ffs(s) - 1 : 0;  // 0: the cell itself, which is fluid
+                f[n] = flag[c.idx(cx(i[n]), cy(i[n]), cz(i[n]))];
+                s &= s - 1u;
+            }
+#pragma unroll
+            for (int n = 0; n < 6; ++n)
+                if (f[n] == FLAG_PART0 + p) d |= 1u << i[n];
         }
-        return m;
+        return d;
     };
+    // directions of the first KEEP cells of the range, for the second pass
+    constexpr int KEEP = 4 * PT;
+    __shared__ unsigned keep[KEEP];
     int mine = 0;
+#pragma unroll 1
     for (int k = lo + (int)threadIdx.x; k < hi; k += PT) {
         unsigned r;
-        mine += __popc(dirs(k, r));
+        const unsigned m = dirs(k, r);
+        if (k - lo < KEEP) keep[k - lo] = m;
+        mine += __popc(m);
     }
     int total_block;
     block_scan(mine, wsum, total_block);
@@ -294,12 +317,22 @@ __device__ __forceinline__ void particle_links(cooperative_groups::cluster_group
     buf ^= 1;
     long long *out = links + seg_begin[seg];
     if (total_block > 0)
+#pragma unroll 1
         for (int k0 = lo; k0 < hi; k0 += PT) {
             const int k = k0 + (int)threadIdx.x;
             unsigned r = 0, m = 0;
-            if (k < hi) m = dirs(k, r);
+            if (k < hi) {
+                if (k - lo >= KEEP) {
+                    m = dirs(k, r);
+                } else if ((m = keep[k - lo]) != 0u) {
+                    int x, y, z;
+                    box_cell(g, w, k, x, y, z);
+                    r = cell_index(g, x, y, z);
+                }
+            }
             int n;
             int pos = base + block_scan(__popc(m), wsum, n);
+#pragma unroll 1
             for (; m; m &= m - 1) {
                 if (pos < cap) out[pos] = ((long long)r << 5) | (__ffs(m) - 1);
                 ++pos;
@@ -312,8 +345,8 @@ __device__ __forceinline__ void particle_links(cooperative_groups::cluster_group
 // Links of the particles marked as changed (set-up and restore).
 template <class S>
 __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
-    k_particle_links(Geo g, const PartDev *parts, const uint8_t *flag, long long *links, const int *seg_begin,
-                     int *seg_count, int first_seg, const int *capacity) {
+    k_particle_links(Geo g, const PartDev *parts, const uint8_t *flag, const uint32_t *mask, long long *links,
+                     const int *seg_begin, int *seg_count, int first_seg, const int *capacity) {
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     __shared__ ClusterCounts counts;
     __shared__ int wsum[PW];
@@ -321,8 +354,8 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
     const int p = (int)blockIdx.x / PC;
     cl.sync();  // every block of the cluster is running before its shared memory is written
     if (parts[p].changed)
-        particle_links<S>(cl, g, parts[p], p, flag, links, seg_begin, seg_count, first_seg + p, capacity[p], counts, buf,
-                          wsum);
+        particle_links(cl, g, parts[p], p, flag, mask, links, seg_begin, seg_count, first_seg + p, capacity[p], counts,
+                       buf, wsum);
     cl.sync();  // no block leaves while another may still write to its shared memory
 }
 
@@ -333,12 +366,23 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
 //   created c:   tau(c) = sum of its stable neighbours' tau / (N_f + 1), each of
 //                them gives up tau(c)/N_f;
 // the deleted / created momentum goes to the particle as an impulse at the cell.
-// The work follows the list (a few cells per step), not the box.
+// The work follows the list (a few cells per step), not the box.  It runs once per launch,
+// so its time is that of dependent loads and of fetching the code: a warp works on one cell
+// (or pair, or mask) with its neighbours, components or directions in the lanes, loads side
+// by side, code rolled up (straight-line code for one thread per cell took 67 us for a
+// single converted cell, where this takes 27 with the masks).
+constexpr int FD_CHUNK = 64, FD_GATHER = 8;  // converted cells per impulse chunk; warps that gather densities
+template <class R>
+struct FillDrainSmem {
+    double pm[FD_CHUNK][6];             // momentum and lever arm of a chunk of converted cells
+    R f[FD_GATHER][(Q - 1) * Q + 2];    // PDFs of a created cell's neighbours, per warp
+};
 template <class S, int PAR>
 __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S> &a, PartDev &P, int p,
-                                           const BoxWalk &w, int nconv, double (*s_pm)[6]) {
+                                           const BoxWalk &w, int nconv, FillDrainSmem<typename Store<S>::R> &sm) {
     using R = typename Store<S>::R;
     constexpr bool SH = Store<S>::shifted;
+    constexpr unsigned ALL = 0xffffffffu;
     const long long np = a.g.np;
     const int nc = w.cells, tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
     R *tau = const_cast<R *>(a.tau);
@@ -350,130 +394,137 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
         if (k >= 0) return kind[k];
         return flag[cell_index(a.g, x, y, z)] == FLAG_FLUID ? 1 : 0;
     };
-    // B: N_f of converted cells, new stress of created cells
-    for (int q = tid; q < nconv; q += PT) {
-        const int k = conv[q], kd = kind[k];
-        int x, y, z, kn[6];
+    // stored location of population i of the cell, in the layout PAR reads
+    auto slot = [&](const Cell &c, int i) -> S * {
+        return PAR == 0 ? a.f + (long long)i * np + c.self()
+                        : a.f + (long long)copp(i) * np + c.idx(-cx(i), -cy(i), -cz(i));
+    };
+    auto outside = [&](int x, int y, int z, int i) -> bool {
+        return (!a.g.per[0] && (x + cx(i) < 0 || x + cx(i) >= a.g.nx)) ||
+               (!a.g.per[1] && (y + cy(i) < 0 || y + cy(i) >= a.g.ny)) ||
+               (!a.g.per[2] && (z + cz(i) < 0 || z + cz(i) >= a.g.nz));
+    };
+    // B: N_f of converted cells, new stress of created cells.  Lane l: face l; then lane c:
+    // component c, summed in face order.
+#pragma unroll 1
+    for (int q = warp; q < nconv; q += PW) {
+        const int k = conv[q];
+        int x, y, z;
         box_cell(a.g, w, k, x, y, z);
-        unsigned nb[6];
+        bool stable = false;
+        unsigned nb = 0;
+        if (lane < 6 && step_cell(a.g, lane, x, y, z)) {
+            stable = kind_of(x, y, z) == 1;
+            nb = cell_index(a.g, x, y, z);
+        }
+        const unsigned sb = __ballot_sync(ALL, stable);
+        const int nf = __popc(sb), c = lane < 6 ? lane : 0;
+        double t[6], sum = 0.0;
 #pragma unroll
         for (int l = 0; l < 6; ++l) {
-            int xq = x, yq = y, zq = z;
-            kn[l] = step_cell(a.g, l, xq, yq, zq) ? kind_of(xq, yq, zq) : 0;
-            nb[l] = cell_index(a.g, xq, yq, zq);
+            const unsigned n = __shfl_sync(ALL, nb, l);
+            t[l] = (sb >> l) & 1u ? (double)tau[c * np + n] : 0.0;
         }
-        int nf = 0;
-        double sum[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
         for (int l = 0; l < 6; ++l)
-            if (kn[l] == 1) {
-                nf++;
-                for (int c = 0; c < 6; ++c) sum[c] += (double)tau[c * np + nb[l]];
-            }
-        nf_arr[k] = (uint8_t)nf;
-        if (kd == 3)
-            for (int c = 0; c < 6; ++c) delta[(long long)c * nc + k] = sum[c] / (double)(nf + 1);
+            if ((sb >> l) & 1u) sum += t[l];
+        if (lane == 0) nf_arr[k] = (uint8_t)nf;
+        if (lane < 6 && kind[k] == 3) delta[(long long)c * nc + k] = sum / (double)(nf + 1);
     }
     __syncthreads();
     // C: stress gathered by each stable cell from its converted D3Q7 neighbours, face by
     // face.  Pair e = (converted cell, face) stands for the stable cell on that face when
-    // the converted cell is the first one in that cell's face order; returns its place in
-    // the box, or -1.
-    auto owned = [&](int e, int &x, int &y, int &z, int (&kb)[6], int (&kk)[6]) -> int {
-        const int q = e / 6, l = e - 6 * q;
-        box_cell(a.g, w, conv[q], x, y, z);
-        if (!step_cell(a.g, l, x, y, z)) return -1;
-        const int ks = box_index(a.g, w, x, y, z);
-        if (ks < 0 || kind[ks] != 1) return -1;
-        int first = -1;
-#pragma unroll
-        for (int m = 0; m < 6; ++m) {
-            int xq = x, yq = y, zq = z;
-            kb[m] = step_cell(a.g, m, xq, yq, zq) ? box_index(a.g, w, xq, yq, zq) : -1;
-            kk[m] = kb[m] >= 0 ? kind[kb[m]] : 0;
-            if (kk[m] < 2) kb[m] = -1;
-            if (first < 0 && kb[m] >= 0) first = kb[m];
-        }
-        return first == conv[q] ? ks : -1;
-    };
-    for (int e = tid; e < 6 * nconv; e += PT) {
-        int x, y, z, kb[6], kk[6];
-        const int ks = owned(e, x, y, z, kb, kk);
-        if (ks < 0) continue;
-        double acc[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-        for (int m = 0; m < 6; ++m) {
-            if (kb[m] < 0) continue;
-            const double nf = (double)nf_arr[kb[m]];
-            if (kk[m] == 2) {
-                int xq = x, yq = y, zq = z;
-                step_cell(a.g, m, xq, yq, zq);
-                const unsigned nb = cell_index(a.g, xq, yq, zq);
-                for (int c = 0; c < 6; ++c) acc[c] += (double)tau[c * np + nb] / nf;
-            } else {
-                for (int c = 0; c < 6; ++c) acc[c] -= delta[(long long)c * nc + kb[m]] / nf;
+    // the converted cell is the first one in that cell's face order.  First pass: the gains,
+    // kept in delta; second pass: added (all gains are formed from the stress before).
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+        for (int e = warp; e < 6 * nconv; e += PW) {
+            const int q = e / 6, l = e - 6 * q;
+            int x, y, z;
+            box_cell(a.g, w, conv[q], x, y, z);
+            if (!step_cell(a.g, l, x, y, z)) continue;
+            const int ks = box_index(a.g, w, x, y, z);
+            if (ks < 0 || kind[ks] != 1) continue;
+            const unsigned r = cell_index(a.g, x, y, z);
+            int kb = -1, kk = 0;
+            unsigned nb = 0;
+            if (lane < 6 && step_cell(a.g, lane, x, y, z)) {
+                kb = box_index(a.g, w, x, y, z);
+                kk = kb >= 0 ? kind[kb] : 0;
+                nb = cell_index(a.g, x, y, z);
             }
+            const unsigned cb = __ballot_sync(ALL, kk >= 2);
+            if (__shfl_sync(ALL, kb, __ffs(cb) - 1) != conv[q]) continue;
+            const int c = lane < 6 ? lane : 0;
+            if (pass == 1) {
+                if (lane < 6) tau[c * np + r] = (R)((double)tau[c * np + r] + delta[(long long)c * nc + ks]);
+                continue;
+            }
+            double acc = 0.0;
+#pragma unroll 1
+            for (unsigned m = cb; m; m &= m - 1u) {
+                const int f = __ffs(m) - 1, kf = __shfl_sync(ALL, kb, f);
+                const unsigned n = __shfl_sync(ALL, nb, f);
+                const bool gone = __shfl_sync(ALL, kk, f) == 2;
+                const double v = gone ? (double)tau[c * np + n] : delta[(long long)c * nc + kf];
+                const double t = v / (double)nf_arr[kf];
+                acc = gone ? acc + t : acc - t;
+            }
+            if (lane < 6) delta[(long long)c * nc + ks] = acc;
         }
-        for (int c = 0; c < 6; ++c) delta[(long long)c * nc + ks] = acc[c];
+        __syncthreads();
     }
     // D: impulses and the populations of created cells, a warp per converted cell: the
     // momentum of a destroyed cell's deleted populations, or f^eq(rho_bar, u_b) written to
     // a created cell with its momentum.  A created cell reads only stable cells' populations
     // and writes only its own, so the cells are independent.  Thread 0 then adds the
     // momenta to the impulse in the sequential order of the method: destroyed cells in cell
-    // order, then created cells in cell order.  Sums over directions run in direction order
-    // (shuffles hand every lane the terms).
+    // order, then created cells in cell order.  Sums over directions run in direction order.
     double dP[3] = {0, 0, 0}, dL[3] = {0, 0, 0};
+    const int i = lane < Q ? lane : 0;  // lane i: population or direction i
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
-        const int want = pass == 0 ? 2 : 3;
-        for (int q0 = 0; q0 < nconv; q0 += PT) {
-            const int m = min(PT, nconv - q0);
-            for (int j = warp; j < m; j += PW) {
+        const int want = pass == 0 ? 2 : 3, warps = pass == 0 ? PW : FD_GATHER;
+#pragma unroll 1
+        for (int q0 = 0; q0 < nconv; q0 += FD_CHUNK) {
+            const int m = min(FD_CHUNK, nconv - q0);
+#pragma unroll 1
+            for (int j = warp; j < m && warp < warps; j += warps) {
                 const int k = conv[q0 + j];
                 if (kind[k] != want) continue;
                 int x, y, z;
                 box_cell(a.g, w, k, x, y, z);
-                const unsigned r = cell_index(a.g, x, y, z);
                 const Cell cl(a.g, x, y, z);
-                double d[3], fi = 0.0;
+                double d[3], fi;
                 min_image(a.g, P.X, x, y, z, d);
                 if (want == 2) {
-                    // lane i: population i
-#pragma unroll
-                    for (int i = 0; i < Q; ++i)
-                        if (lane == i) {
-                            const S *src = PAR == 0 ? a.f + (long long)i * np + r
-                                                    : a.f + (long long)copp(i) * np + cl.idx(-cx(i), -cy(i), -cz(i));
-                            fi = (double)Store<S>::ld(src, a.ph.inv_scale) + (SH ? wgt<double>(i) * (double)a.ph.rho0 : 0.0);
-                        }
+                    fi = (double)Store<S>::ld(slot(cl, i), a.ph.inv_scale) +
+                         (SH ? wgt<double>(i) * (double)a.ph.rho0 : 0.0);
                 } else {
-                    // lane i: density of the neighbour r + c_i if it is stable
+                    // density of the neighbour r + c_i if it is stable
+                    const int xq = cl.X(cx(i)), yq = cl.Y(cy(i)), zq = cl.Z(cz(i));
+                    const bool stable = lane >= 1 && lane < Q && !outside(x, y, z, i) && kind_of(xq, yq, zq) == 1;
+                    const unsigned sb = __ballot_sync(ALL, stable);
+                    R *sf = sm.f[warp];
+#pragma unroll 4
+                    for (int t = lane; t < (Q - 1) * Q; t += 32) {
+                        const int h = 1 + t / Q, pop = t - (h - 1) * Q;
+                        const Cell cn(a.g, cl.X(cx(h)), cl.Y(cy(h)), cl.Z(cz(h)));
+                        sf[t] = (sb >> h) & 1u ? Store<S>::ld(slot(cn, pop), a.ph.inv_scale) : R(0);
+                    }
+                    __syncwarp();
                     double rn = 0.0;
-                    bool stable = false;
-                    int xq = x, yq = y, zq = z;
-                    if (lane >= 1 && lane < Q) {
-                        const int dx = cx(lane), dy = cy(lane), dz = cz(lane);
-                        const bool out = (!a.g.per[0] && (x + dx < 0 || x + dx >= a.g.nx)) ||
-                                         (!a.g.per[1] && (y + dy < 0 || y + dy >= a.g.ny)) ||
-                                         (!a.g.per[2] && (z + dz < 0 || z + dz >= a.g.nz));
-                        if (!out) {
-                            xq = cl.X(dx);
-                            yq = cl.Y(dy);
-                            zq = cl.Z(dz);
-                            stable = kind_of(xq, yq, zq) == 1;
-                        }
-                    }
-                    if (stable) {
-                        const Cell cn(a.g, xq, yq, zq);
-                        R fn[Q];
-                        load_pdfs<S, PAR>(a, cn, cn.self(), fn);
-                        for (int i = 0; i < Q; ++i) rn += (double)fn[i] + (SH ? wgt<double>(i) * (double)a.ph.rho0 : 0.0);
-                    }
-                    const unsigned sb = __ballot_sync(0xffffffffu, stable);
+                    if (stable)
+#pragma unroll 1
+                        for (int pop = 0; pop < Q; ++pop)
+                            rn += (double)sf[(lane - 1) * Q + pop] + (SH ? wgt<double>(pop) * (double)a.ph.rho0 : 0.0);
+                    __syncwarp();
                     double rsum = 0.0;
-                    for (int i = 1; i < Q; ++i) {
-                        const double t = __shfl_sync(0xffffffffu, rn, i);
-                        if ((sb >> i) & 1u) rsum += t;
+#pragma unroll 1
+                    for (int h = 1; h < Q; ++h) {
+                        const double t = __shfl_sync(ALL, rn, h);
+                        if ((sb >> h) & 1u) rsum += t;
                     }
                     const int cnt = __popc(sb);
                     const double rho_bar = cnt > 0 ? rsum / (double)cnt : (double)a.ph.rho_ref;
@@ -482,68 +533,56 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
                                            P.w[0] * d[1] - P.w[1] * d[0]};
                     for (int c3 = 0; c3 < 3; ++c3) ub[c3] = P.v[c3] + wxd[c3];
                     const double usq = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
-#pragma unroll
-                    for (int i = 0; i < Q; ++i)
-                        if (lane == i) {
-                            const double cu = cx(i) * ub[0] + cy(i) * ub[1] + cz(i) * ub[2];
-                            fi = wgt<double>(i) * rho_bar * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * usq);
-                            S *dst = PAR == 0 ? a.f + (long long)i * np + r
-                                              : a.f + (long long)copp(i) * np + cl.idx(-cx(i), -cy(i), -cz(i));
-                            const double v = SH ? fi - wgt<double>(i) * (double)a.ph.rho0 : fi;
-                            Store<S>::st(dst, (R)v, a.ph.scale);
-                        }
+                    const double cu = cx(i) * ub[0] + cy(i) * ub[1] + cz(i) * ub[2];
+                    fi = wgt<double>(i) * rho_bar * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * usq);
+                    if (lane < Q) {
+                        const double v = SH ? fi - wgt<double>(i) * (double)a.ph.rho0 : fi;
+                        Store<S>::st(slot(cl, i), (R)v, a.ph.scale);
+                    }
                 }
                 double Pm = 0.0;  // lanes 0..2: the momentum's components
-                for (int i = 0; i < Q; ++i) {
-                    const double t = __shfl_sync(0xffffffffu, fi, i);
-                    Pm += t * (double)cdir(i, lane % 3);
+#pragma unroll 1
+                for (int h = 0; h < Q; ++h) {
+                    const double t = __shfl_sync(ALL, fi, h);
+                    Pm += t * (double)cdir(h, lane % 3);
                 }
-                if (lane < 3) s_pm[j][lane] = Pm;
+                if (lane < 3) sm.pm[j][lane] = Pm;
                 if (lane == 0)
-                    for (int c3 = 0; c3 < 3; ++c3) s_pm[j][3 + c3] = d[c3];
+                    for (int c3 = 0; c3 < 3; ++c3) sm.pm[j][3 + c3] = d[c3];
             }
             __syncthreads();
             if (tid == 0) {
+#pragma unroll 1
                 for (int t = 0; t < m; ++t) {
                     const int k = conv[q0 + t];
                     if (kind[k] != want) continue;
-                    const double *Pm = s_pm[t], *d = s_pm[t] + 3;
-                    if (want == 2) {
-                        dP[0] += Pm[0];
-                        dP[1] += Pm[1];
-                        dP[2] += Pm[2];
-                        dL[0] += d[1] * Pm[2] - d[2] * Pm[1];
-                        dL[1] += d[2] * Pm[0] - d[0] * Pm[2];
-                        dL[2] += d[0] * Pm[1] - d[1] * Pm[0];
-                        if (nf_arr[k] == 0) {
-                            int x, y, z;
-                            box_cell(a.g, w, k, x, y, z);
-                            const unsigned r = cell_index(a.g, x, y, z);
-                            for (int c = 0; c < 6; ++c) E.diag[c] += (double)tau[c * np + r];
-                        }
-                        E.diag[6] += 1.0;
-                    } else {
-                        dP[0] -= Pm[0];
-                        dP[1] -= Pm[1];
-                        dP[2] -= Pm[2];
-                        dL[0] -= d[1] * Pm[2] - d[2] * Pm[1];
-                        dL[1] -= d[2] * Pm[0] - d[0] * Pm[2];
-                        dL[2] -= d[0] * Pm[1] - d[1] * Pm[0];
-                        E.diag[7] += 1.0;
+                    const double *Pm = sm.pm[t], *d = sm.pm[t] + 3;
+                    const double s = want == 2 ? 1.0 : -1.0;  // x + s y: exactly x + y or x - y
+                    dP[0] += s * Pm[0];
+                    dP[1] += s * Pm[1];
+                    dP[2] += s * Pm[2];
+                    dL[0] += s * (d[1] * Pm[2] - d[2] * Pm[1]);
+                    dL[1] += s * (d[2] * Pm[0] - d[0] * Pm[2]);
+                    dL[2] += s * (d[0] * Pm[1] - d[1] * Pm[0]);
+                    if (want == 2 && nf_arr[k] == 0) {
+                        int x, y, z;
+                        box_cell(a.g, w, k, x, y, z);
+                        const unsigned r = cell_index(a.g, x, y, z);
+                        for (int c = 0; c < 6; ++c) E.diag[c] += (double)tau[c * np + r];
                     }
+                    E.diag[want == 2 ? 6 : 7] += 1.0;
                 }
             }
             __syncthreads();
         }
     }
-    // E: apply the stress moves, then the converted cells' stress and flags
-    for (int e = tid; e < 6 * nconv; e += PT) {
-        int x, y, z, kb[6], kk[6];
-        const int ks = owned(e, x, y, z, kb, kk);
-        if (ks < 0) continue;
-        const unsigned r = cell_index(a.g, x, y, z);
-        for (int c = 0; c < 6; ++c) tau[c * np + r] = (R)((double)tau[c * np + r] + delta[(long long)c * nc + ks]);
-    }
+    if (tid == 0)
+        for (int c3 = 0; c3 < 3; ++c3) {
+            P.dP[c3] = dP[c3];
+            P.dL[c3] = dL[c3];
+        }
+    // E: the converted cells' stress and flags
+#pragma unroll 1
     for (int q = tid; q < nconv; q += PT) {
         const int k = conv[q];
         int x, y, z;
@@ -556,27 +595,27 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
     }
     __syncthreads();
     // F: neighbour masks of the converted cells and their neighbours (the only cells whose
-    // masks change; a cell reached twice gets the same value twice)
-    for (int e = tid; e < nconv * Q; e += PT) {
-        const int q = e / Q, i = e - q * Q;
+    // masks change; a cell reached twice gets the same value twice): a warp per mask, lane i
+    // looking in direction i (see cell_mask)
+#pragma unroll 1
+    for (int e = warp; e < nconv * Q; e += PW) {
+        const int q = e / Q, h = e - q * Q;
         int x, y, z;
         box_cell(a.g, w, conv[q], x, y, z);
-        if ((!a.g.per[0] && (x + cx(i) < 0 || x + cx(i) >= a.g.nx)) ||
-            (!a.g.per[1] && (y + cy(i) < 0 || y + cy(i) >= a.g.ny)) ||
-            (!a.g.per[2] && (z + cz(i) < 0 || z + cz(i) >= a.g.nz)))
-            continue;
-        const Cell cl(a.g, x, y, z);
-        const int xq = cl.X(cx(i)), yq = cl.Y(cy(i)), zq = cl.Z(cz(i));
-        E.mask[cell_index(a.g, xq, yq, zq)] = cell_mask(a.g, flag, xq, yq, zq);
+        if (outside(x, y, z, h)) continue;
+        const Cell c0(a.g, x, y, z);
+        const Cell c1(a.g, c0.X(cx(h)), c0.Y(cy(h)), c0.Z(cz(h)));
+        int fl = FLAG_FLUID;
+        if (lane < Q)
+            fl = outside(c1.x, c1.y, c1.z, lane) ? FLAG_NOSLIP : flag[c1.idx(cx(lane), cy(lane), cz(lane))];
+        uint32_t m = __ballot_sync(ALL, fl != FLAG_FLUID);
+        if (__ballot_sync(ALL, lane > 0 && fl != FLAG_FLUID && fl != FLAG_NOSLIP)) m |= MASK_MOVING;
+        if (lane == 0) E.mask[c1.self()] = m;
     }
-    if (tid == 0) {
-        P.changed = 1;
-        for (int c3 = 0; c3 < 3; ++c3) {
-            P.dP[c3] = dP[c3];
-            P.dL[c3] = dL[c3];
-            P.v[c3] += dP[c3] / P.m;
-            P.w[c3] += dL[c3] / P.I;
-        }
+    if (tid < 3) {
+        if (tid == 0) P.changed = 1;
+        P.v[tid] += P.dP[tid] / P.m;
+        P.w[tid] += P.dL[tid] / P.I;
     }
     __syncthreads();
 }
@@ -588,9 +627,10 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
 // Every cell of a particle's box is classified each step and few convert, so
 // the bounds are latency and the FP64 pipe: the cluster spreads the classification and the
 // link list over PC x PT threads and as many SMs, FP64 work runs in single threads or in
-// lanes side by side, and the conversions work on a list.  Before, three kernels of one
-// block each took 40 us per step of an R = 8 sphere without conversions and about 300
-// with them.
+// lanes side by side, and the conversions work on a list.  An R = 8 sphere takes 18 us per
+// step without conversions (11 of them the classification with the surface velocities) and
+// 66 with one converted cell (16 of them the links); three kernels of one block each took
+// 40 and about 300.
 // One cluster per solve: entries[blockIdx.x / PC], or `one` when entries is nullptr.
 template <class S>
 __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
@@ -605,7 +645,7 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
     __shared__ int wsum[PW], s_mine;
     __shared__ BoxWalk w;
     __shared__ SphereFilter sf;
-    __shared__ double s_pm[PT][6];  // momentum and lever arm of a chunk of converted cells
+    __shared__ FillDrainSmem<typename Store<S>::R> sm;
     int buf = 0;
     if (rank == 0) {
         if (E.sums) {
@@ -640,24 +680,27 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
     for (int p = 0; p < E.nparts; ++p) {
         PartDev &P = E.parts[p];
         __syncthreads();
-        if (tid == 0) {
-            w = box_walk(a.g, particle_bbox(a.g, P.X, P.R, 3));
-            sf = sphere_filter(a.g, P);
-            s_mine = 0;
-        }
+        if (warp == 0) prepare_box(a.g, P, 3, w, &sf);
+        if (tid == 0) s_mine = 0;
         __syncthreads();
         // A: classify a consecutive range of the box
         const int per = (w.cells + PC - 1) / PC, lo = min(w.cells, per * rank), hi = min(w.cells, lo + per);
         int mine = 0;
-#pragma unroll 4
+#pragma unroll 1
         for (int q = lo + tid; q < hi; q += PT) {
             int x, y, z;
             box_cell(a.g, w, q, x, y, z);
-            const int old = E.flag[cell_index(a.g, x, y, z)];
+            const unsigned r = cell_index(a.g, x, y, z);
+            const int old = E.flag[r];
             int kd = 0;
             if (old == FLAG_FLUID || old == FLAG_PART0 + p) {
-                const bool inside = inside_sphere(a.g, P, sf, x, y, z);
+                float d2;
+                const bool inside = inside_sphere(a.g, P, sf, x, y, z, d2);
                 kd = old == FLAG_FLUID ? (inside ? 2 : 1) : (inside ? 0 : 3);
+                // the surface velocity of a cell the sphere keeps (again below when
+                // conversions change the sphere's velocity).  A cell deeper than sqrt(2)
+                // below the surface has no fluid neighbour to read it.
+                if (kd == 0 && d2 >= sf.deep2) set_solid_velocity<S>(a, x, y, z, r, a.u_out, a.u_out);
             }
             E.kind[q] = (uint8_t)kd;
             mine += kd >= 2 ? 1 : 0;
@@ -688,28 +731,33 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
         cl.sync();
         if (rank == 0) {
             if (((E.parity0 + k) & 1) == 0)
-                fill_drain<S, 0>(E, a, P, p, w, nconv, s_pm);
+                fill_drain<S, 0>(E, a, P, p, w, nconv, sm);
             else
-                fill_drain<S, 1>(E, a, P, p, w, nconv, s_pm);
+                fill_drain<S, 1>(E, a, P, p, w, nconv, sm);
         }
         cl.sync();
     }
-    // the spheres' surface velocities, by the state the next step works with
-    for (int p = 0; p < E.nparts; ++p) {
-        __syncthreads();
-        if (tid == 0) w = box_walk(a.g, particle_bbox(a.g, E.parts[p].X, E.parts[p].R, 3));
-        __syncthreads();
+    // surface velocities of the spheres whose velocity the conversions changed
+    for (int p = E.nparts - 1; p >= 0; --p) {
+        if (!((changed >> p) & 1ull)) continue;
+        if (p + 1 < E.nparts) {  // the box of the last particle is still there
+            __syncthreads();
+            if (warp == 0) prepare_box(a.g, E.parts[p], 3, w, nullptr);
+            __syncthreads();
+        }
+#pragma unroll 1
         for (int q = rank * PT + tid; q < w.cells; q += PC * PT) {
             int x, y, z;
             box_cell(a.g, w, q, x, y, z);
             const unsigned r = cell_index(a.g, x, y, z);
-            if (E.flag[r] == FLAG_PART0 + p) set_solid_velocity<S>(a, x, y, z, r, a.u_out, a.u_out);
+            if (E.flag[r] == FLAG_PART0 + p && (E.mask[r] & 0x7fffeu) != 0x7fffeu)
+                set_solid_velocity<S>(a, x, y, z, r, a.u_out, a.u_out);
         }
     }
     for (int p = 0; p < E.nparts; ++p)
         if ((changed >> p) & 1ull)
-            particle_links<S>(cl, a.g, E.parts[p], p, E.flag, E.links, E.seg_begin, E.seg_count, E.first_seg + p,
-                              E.capacity[p], counts, buf, wsum);
+            particle_links(cl, a.g, E.parts[p], p, E.flag, E.mask, E.links, E.seg_begin, E.seg_count, E.first_seg + p,
+                           E.capacity[p], counts, buf, wsum);
     cl.sync();  // no block leaves while another may still write to its shared memory
 }
 

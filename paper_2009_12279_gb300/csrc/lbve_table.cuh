@@ -363,8 +363,8 @@ struct Launch {
     static cudaError_t particle_links(const DevState &d, int nparts, long long *links, const int *seg_begin,
                                       int *seg_count, int first_seg, const int *capacity, cudaStream_t s) {
         if (nparts <= 0) return cudaSuccess;
-        k_particle_links<S><<<nparts * PC, PT, 0, s>>>(d.g, d.parts, d.flag, links, seg_begin, seg_count, first_seg,
-                                                       capacity);
+        k_particle_links<S><<<nparts * PC, PT, 0, s>>>(d.g, d.parts, d.flag, d.mask, links, seg_begin, seg_count,
+                                                       first_seg, capacity);
         return cudaGetLastError();
     }
     static cudaError_t build_mask_impl(const DevState &d, int lx, int ly, int lz, int ex, int ey, int ez,
