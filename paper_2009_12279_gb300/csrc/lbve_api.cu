@@ -568,6 +568,7 @@ lbve_status create_impl(const lbve_params *p, void *stream, lbve_alloc_fn alloc,
     g.n = (long long)p->nx * p->ny * p->nz;
     g.np = padded(g.n);
     c->d.block_x = lbve::default_block_x(*p);
+    c->d.sms = device_sms();
     c->d.auto_kernels = p->schedule == LBVE_SCHED_AUTO ? 1 : (p->schedule == LBVE_SCHED_PIPELINED ? 2 : 0);
     if (p->block_x == 0) {  // a schedule tuned for this shape earlier in the process
         int bx = 0, zc = 0;

@@ -58,6 +58,14 @@ inline int resident_blocks(K kernel, int threads, size_t smem) {
     return sms * per;
 }
 
+inline int device_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        cudaGetLastError();
+    return sms;
+}
+
 // True when the stream is being captured (or its state cannot be asked for): the plain
 // launches are recorded then.
 inline bool capturing(cudaStream_t s) {

@@ -23,9 +23,11 @@ namespace lbve {
 // neighbour addresses live and drops to ~10 % occupancy.  Measured at 512^3: FP32 runs
 // fastest at 7 blocks (72 registers; 8 blocks spill more, 9 or more lose); with the
 // stochastically rounded 16-bit stores BF16 at 7 (4.00 ms against 4.03 at 8) and FP16 at
-// 8 (4.03 ms against 4.09 at 7); FP64 keeps 8.
+// 8 (4.03 ms against 4.09 at 7); FP64, bound by its pipe from a few warps on, at 4 (no
+// spills).
 template <class S, int PAR>
 constexpr int lb_min_blocks() {
+    if (sizeof(S) == 8) return 4;
     return (sizeof(S) == 4 || std::is_same<S, __nv_bfloat16>::value) ? 7 : 8;
 }
 // 256-thread stress blocks, 3 resident per SM (80 registers: no spills at 4)
@@ -293,7 +295,7 @@ __device__ __forceinline__ void lb_cell_at(const KArgs<S> &a, int x, int y, int 
 #pragma unroll
     for (int c = 0; c < 6; ++c) tr[c] = a.tq[c][r];
     const uint32_t m = a.mask[r];
-    step_next();
+    if constexpr (Store<S>::shifted) step_next();
     if (m & 1u) return;
     auto tn = [&](int l, int c) -> R {
         const int k = l >> 1, s = (l & 1) ? -1 : 1;
@@ -324,7 +326,7 @@ __device__ __forceinline__ void fv_cell_at(const KArgs<S> &a, int x, int y, int 
 #pragma unroll
     for (int j = 0; j < 3; ++j) ur[j] = a.uiq[j][r];
     const uint32_t m = a.mask[r];
-    step_next();
+    if constexpr (Store<S>::shifted) step_next();
     if (m & 1u) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) out[c] = R(0);
@@ -794,16 +796,13 @@ __device__ __forceinline__ void fv_tile(const KArgs<S> &a, FvSmem<typename Store
     for (int z = z0; z < z1; ++z) {
         const uint32_t m = m_next;
         if (own && z + 1 < z1) m_next = a.mask[(unsigned)x + nx * (unsigned)y + nxy * (unsigned)(z + 1)];
-        // plane z + 1 + AHEAD is fetched while plane z is updated (an empty group keeps
-        // the count); it goes to the slot of plane z - 2, free since the barrier that
-        // ended the previous plane; planes up to z + 1 have landed
-        if (z + 1 + LBVE_FV_AHEAD <= z1)
-            stage(z + 1 + LBVE_FV_AHEAD);
-        else
-            cp_async_commit();
-        if (z + 1 == z1) step_next();
-        asm volatile("cp.async.wait_group %0;\n" ::"n"(LBVE_FV_AHEAD) : "memory");
+        // planes up to z + 1 have landed; behind the barrier plane z - 1 is done with in the
+        // whole block, so plane z + 1 + AHEAD may take the slot of plane z - 2 and arrives
+        // while plane z is updated: one barrier per plane
+        cp_async_wait_all();
         __syncthreads();
+        if (z + 1 + LBVE_FV_AHEAD <= z1) stage(z + 1 + LBVE_FV_AHEAD);
+        if (z + 1 == z1) step_next();
         if (own) {
             const unsigned r = (unsigned)x + nx * (unsigned)y + nxy * (unsigned)z;
             R out[6];
@@ -823,9 +822,7 @@ __device__ __forceinline__ void fv_tile(const KArgs<S> &a, FvSmem<typename Store
 #pragma unroll
             for (int c = 0; c < 6; ++c) tau_out(c)[r] = out[c];
         }
-        __syncthreads();  // the next stage overwrites the slot of plane z - 1
     }
-    cp_async_wait_all();
 }
 
 template <class S, bool VAR, bool ZR = false, bool W16 = false>
@@ -918,13 +915,11 @@ __global__ void __launch_bounds__(FP_NT, 2) k_fv_pair(KArgs<S> a, int zchunk) {
     for (int z = z0; z < z1; ++z) {
         const uint2 m = m_next;
         if (own && z + 1 < z1) m_next = mask2(z + 1);
-        if (z + 1 + LBVE_FV_AHEAD <= z1)
-            stage(z + 1 + LBVE_FV_AHEAD);
-        else
-            cp_async_commit();
-        if (z + 1 == z1) step_next();
-        asm volatile("cp.async.wait_group %0;\n" ::"n"(LBVE_FV_AHEAD) : "memory");
+        // one barrier per plane, as in fv_tile
+        cp_async_wait_all();
         __syncthreads();
+        if (z + 1 + LBVE_FV_AHEAD <= z1) stage(z + 1 + LBVE_FV_AHEAD);
+        if (z + 1 == z1) step_next();
         if (own) {
             const unsigned r = (unsigned)x + nxu * (unsigned)y + nxy * (unsigned)z;
             const bool fa = !(m.x & 1u), fb = !(m.y & 1u);
@@ -971,9 +966,7 @@ __global__ void __launch_bounds__(FP_NT, 2) k_fv_pair(KArgs<S> a, int zchunk) {
 #pragma unroll
             for (int c = 0; c < 6; ++c) *reinterpret_cast<float2 *>(a.toq[c] + r) = out[c];
         }
-        __syncthreads();  // the next stage overwrites the slot of plane z - 1
     }
-    cp_async_wait_all();
 }
 
 // ---------------------------------------------------------------------------------
@@ -1302,20 +1295,26 @@ __global__ void k_init(KArgs<S> a, const double *__restrict__ rho_in, const doub
     for (int c = 0; c < 6; ++c) tau_dst[c * a.g.np + r] = (R)t6[c];
 }
 
-// rho, physical u and tau of the cells in z-planes z0.. (grid z extent), 0 in non-fluid
-// cells; FP64 outputs indexed from the slab's first cell r0 with leading dimension ld.
-template <class S, int PAR>
-__global__ void k_read(KArgs<S> a, double *__restrict__ rho_out, double *__restrict__ u_out,
-                       double *__restrict__ tau_out, int z0, long long ld) {
+// rho, physical u and tau of the a.lin cells from plane a.zlo on, 0 in non-fluid cells;
+// FP64 outputs indexed from the first of them with leading dimension ld.
+template <class S, int PAR, bool LIN>
+__global__ void __launch_bounds__(128) k_read(KArgs<S> a, double *__restrict__ rho_out, double *__restrict__ u_out,
+                                              double *__restrict__ tau_out, long long ld) {
     using R = typename Store<S>::R;
     constexpr bool SH = Store<S>::shifted;
     step_wait();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= a.g.nx) return;
-    const Cell cl(a.g, x, blockIdx.y, blockIdx.z + z0);
+    int x, y, z;
+    if (!cell_of_thread<S, LIN>(a, x, y, z)) return;
+    const Cell cl(a.g, x, y, z);
     const unsigned r = cl.self();
-    const long long k = (long long)r - (long long)z0 * a.g.nx * a.g.ny;
-    if (a.flag[r] != FLAG_FLUID) {
+    const long long k = (long long)r - (long long)a.zlo * a.g.nx * a.g.ny;
+    // the loads go out together with the mask, as in the stream-collide
+    R f[Q], tr[6];
+    load_pdfs<S, PAR>(a, cl, r, f);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) tr[c] = a.tq[c][r];
+    const uint32_t m = a.mask[r];
+    if (m & 1u) {
         if (rho_out) rho_out[k] = 0.0;
         for (int j = 0; j < 3; ++j)
             if (u_out) u_out[j * ld + k] = 0.0;
@@ -1323,23 +1322,25 @@ __global__ void k_read(KArgs<S> a, double *__restrict__ rho_out, double *__restr
             if (tau_out) tau_out[c * ld + k] = 0.0;
         return;
     }
-    R f[Q];
-    load_pdfs<S, PAR>(a, cl, r, f);
+    auto tn = [&](int l, int c) -> R {
+        const int q = l >> 1, s = (l & 1) ? -1 : 1;
+        return a.tq[c][cl.idx(q == 0 ? s : 0, q == 1 ? s : 0, q == 2 ? s : 0)];
+    };
     R Fp[3], F[3], u[3], rho, drho;
-    polymer_force<R>(a.g, a.ph, cl, r, a.mask[r], a.tau, Fp);
+    if (a.ph.fene)
+        polymer_force_core_fene<R>(tr, m, tn, a.ph, Fp);
+    else
+        polymer_force_core<R>(tr, m, tn, Fp);
 #pragma unroll
     for (int j = 0; j < 3; ++j) F[j] = a.ph.g[j] + Fp[j];
     moments<R, SH>(f, F, a.ph.rho0, rho, drho, u);
     if (rho_out) rho_out[k] = SH ? (double)a.ph.rho0 + (double)drho : (double)rho;
-    for (int j = 0; j < 3; ++j)
-        if (u_out) u_out[j * ld + k] = (double)u[j];
-    if (tau_out) {
-        R t6[6];
+    if (u_out)
 #pragma unroll
-        for (int c = 0; c < 6; ++c) t6[c] = a.tau[c * a.g.np + r];
+        for (int j = 0; j < 3; ++j) u_out[j * ld + k] = (double)u[j];
+    if (tau_out)
 #pragma unroll
-        for (int c = 0; c < 6; ++c) tau_out[c * ld + k] = (double)stored_to_stress<R>(a.ph, t6, c);
-    }
+        for (int c = 0; c < 6; ++c) tau_out[c * ld + k] = (double)stored_to_stress<R>(a.ph, tr, c);
 }
 
 // PDFs of every cell to / from unshifted FP64 in the plain (pre-collision) layout.

@@ -104,6 +104,7 @@ struct DevState {
     // 1: the step's kernels are launched as programmatic dependents of one another (see
     // launch_step); 0: plain launches (pools, phases, captured streams)
     int pdl = 0;
+    int sms = 0;  // SMs of the device (0: asked for when needed)
 };
 
 #ifdef __CUDACC__
@@ -114,7 +115,7 @@ __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;
 // ... and lets its own successor be launched once all its blocks have come here.  After
 // a block's loads, not at its start: blocks that wait from early on take the slots of, and
 // were measured to spread unevenly among, those at work (FP64 32^3: 185 us per step instead
-// of 65).
+// of 65).  FP64 kernels, whose time is arithmetic, leave it to their blocks' ends.
 __device__ __forceinline__ void step_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 

@@ -119,6 +119,7 @@ lbve_status lbve_step_noalloc(const lbve_params *p, void *f, void *tau_a, void *
     d.parts = (PartDev *)parts;
     d.cur = 0;
     d.block_x = default_block_x(*p);
+    d.sms = device_sms();
     d.fv_zchunk = 0;
     // AUTO: the stress kernel small grids take (the large-grid kernels start beyond the cell limit)
     d.auto_kernels = p->schedule == LBVE_SCHED_AUTO ? 1 : 0;

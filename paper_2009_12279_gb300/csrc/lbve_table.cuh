@@ -171,13 +171,22 @@ struct Launch {
     // measured on GB300 (stream-collide, event-timed, FP32, nx x 64 x 64, tiles against
     // order) 33: 12.3 / 10.3 us, 110: 20.2 / 19.5, 120: 19.4 / 20.8, 240: 42.0 / 43.8; BF16
     // 165: 26.5 / 25.5.  The line lies at 7/8 of the lanes in use.
-    template <class K>
-    static cudaError_t cell_launch(const DevState &d, K tiled, K linear, cudaStream_t s) {
+    template <class K, class... A>
+    static cudaError_t cell_launch(const DevState &d, K tiled, K linear, cudaStream_t s, A... more) {
         const KArgs<S> a = args(d);
+        // grids with less than a 128-thread block per SM: smaller blocks in memory order, so
+        // that the cells spread over the SMs (an SM issues a warp's FP64 instruction in 16
+        // cycles, whatever the number of warps waiting: FP64 4 x 32 x 4 on 4 SMs 35.5 us per
+        // step, on 16 27.7)
+        const unsigned sms = (unsigned)(d.sms > 0 ? d.sms : sm_count());
+        if (a.lin <= 96u * sms) {
+            const unsigned t = std::max(32u, (a.lin / sms + 31u) / 32u * 32u);
+            return launch_step(d.pdl, linear, dim3((a.lin + t - 1u) / t), dim3(t), 0, s, a, more...);
+        }
         const dim3 b = block2(d), g = grid2(d);
         if (8LL * d.g.nx * d.g.ny >= 7LL * g.x * b.x * g.y * b.y)
-            return launch_step(d.pdl, tiled, g, b, 0, s, a);
-        return launch_step(d.pdl, linear, dim3((a.lin + 127u) / 128u), dim3(128), 0, s, a);
+            return launch_step(d.pdl, tiled, g, b, 0, s, a, more...);
+        return launch_step(d.pdl, linear, dim3((a.lin + 127u) / 128u), dim3(128), 0, s, a, more...);
     }
     static cudaError_t lb(const DevState &d, int parity, cudaStream_t s) {
         if (d.auto_kernels && rows_ok(d)) return lb_rows(d, parity, s);
@@ -397,11 +406,11 @@ struct Launch {
     static cudaError_t read(const DevState &d, int parity, double *rho, double *u, double *tau, int z0, int z1,
                             long long ld, cudaStream_t s) {
         if (z1 <= z0) return cudaSuccess;
-        KArgs<S> a = args(d);
-        dim3 g = grid3(d);
-        g.z = (unsigned)(z1 - z0);
-        return launch_step(d.pdl, parity == 0 ? k_read<S, 0> : k_read<S, 1>, g, dim3(d.block_x), 0, s, a, rho, u, tau, z0,
-                           ld);
+        DevState q = d;
+        q.zlo = z0;
+        q.zhi = z1;
+        return parity == 0 ? cell_launch(q, k_read<S, 0, false>, k_read<S, 0, true>, s, rho, u, tau, ld)
+                           : cell_launch(q, k_read<S, 1, false>, k_read<S, 1, true>, s, rho, u, tau, ld);
     }
     static cudaError_t pdfs_io(const DevState &d, int parity, double *io, int write, cudaStream_t s) {
         KArgs<S> a = args(d);
