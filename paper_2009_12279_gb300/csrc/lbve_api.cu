@@ -378,8 +378,8 @@ void prefault_output(void *p, size_t bytes) {
     b[bytes - 1] = 0;
 }
 
-// Advance a pool's device step counter (after each step's stream-collide).
-__global__ void k_step_count(unsigned *dstep) { *dstep += 1u; }
+// Advance a pool's device step counter (after each step's stream-collide, or after a call).
+__global__ void k_step_count(unsigned *dstep, unsigned n) { *dstep += n; }
 
 PartScratch part_scratch(const lbve_ctx *c) {
     PartScratch ps;
@@ -1376,15 +1376,18 @@ static int residual_blocks(const lbve_ctx *c) {
     return (int)(b > 1024 ? 1024 : (b < 1 ? 1 : b));
 }
 
-static lbve_status residual_enqueue(lbve_ctx *c) {
+// Block partials of the residual into `partial` (nullptr: the context's own buffer) on a
+// stream that follows the context's.
+static lbve_status residual_enqueue(lbve_ctx *c, double *partial = nullptr, cudaStream_t st = nullptr) {
     const int nb = residual_blocks(c);
+    if (!partial) st = c->stream;
     if (!c->usnap) {
         c->usnap = dev_alloc(c, (size_t)3 * c->d.g.np * c->kt->real_bytes);
         c->res_partial = (double *)dev_alloc(c, sizeof(double) * 2 * 1024);
         if (!c->usnap || !c->res_partial) return fail(c, LBVE_ENOMEM, "residual buffers");
-        CK(cudaMemsetAsync(c->usnap, 0, (size_t)3 * c->d.g.np * c->kt->real_bytes, c->stream), "residual clear");
+        CK(cudaMemsetAsync(c->usnap, 0, (size_t)3 * c->d.g.np * c->kt->real_bytes, st), "residual clear");
     }
-    CK(c->kt->residual(c->d, c->usnap, c->res_partial, nb, c->stream), "residual kernel");
+    CK(c->kt->residual(c->d, c->usnap, partial ? partial : c->res_partial, nb, st), "residual kernel");
     return LBVE_OK;
 }
 
@@ -1469,7 +1472,11 @@ struct lbve_pool {
     int n_pentries = 0;
     int total_lb = 0;
     int grid_lb = 0;
-    unsigned *dstep = nullptr;  // device: steps since the entries were built
+    unsigned *dstep = nullptr;  // device: [0] steps since the entries were built, [1] the same
+                                // at the start of the call
+    // Members with kernels of their own (see enqueue_steps), the largest first, and the
+    // members of the batched kernels; split when the entries are built
+    std::vector<lbve_ctx *> own, batch;
     struct FvGroup {
         int tx, start, n, total, grid;  // stress tile width, first entry, entries, items, grid
         int var;                        // 1 when a member of the group uses a finite-volume variant
@@ -1516,11 +1523,32 @@ void drop_graphs(lbve_pool *P) {
     }
 }
 
+bool pool_graphs(const lbve_pool *P) {
+    // the legacy default stream cannot be captured: launch directly there
+    return P->use_graphs && (uintptr_t)P->stream > 1;
+}
+
+// Members with kernels of their own in a pool that replays graphs: all of them up to
+// kSide members, those of 2^16 cells and more beyond.  The batched kernels read every
+// parameter and pointer from shared memory and share one shape over all grids (48 members
+// of the serving mix, 13 M cells, BF16: 910 us per step, own kernels on parallel branches
+// of the graph 685; 4 small members 45 and 27 us); launches for many small members would
+// add up.
+constexpr long long kOwnCells = 1LL << 16;
+bool own_kernels(const lbve_pool *P, const lbve_ctx *c) {
+    return pool_graphs(P) && (P->members.size() <= (size_t)lbve_pool::kSide || c->d.g.n >= kOwnCells);
+}
+
 // Entries for the two parities of the call (state after an even / odd number of steps
 // since the build), uploaded once per membership change.
 lbve_status build_entries(lbve_pool *P) {
+    P->own.clear();
+    P->batch.clear();
+    for (lbve_ctx *c : P->members) (own_kernels(P, c) ? P->own : P->batch).push_back(c);
+    std::stable_sort(P->own.begin(), P->own.end(),
+                     [](const lbve_ctx *a, const lbve_ctx *b) { return a->d.g.n > b->d.g.n; });
     const size_t eb = P->kt->batch_entry_bytes;
-    const size_t n = P->members.size();
+    const size_t n = P->batch.size();
     if (n > P->entries_cap) {
         for (int k = 0; k < 2; ++k) {
             if (P->entries[k]) cudaFree(P->entries[k]);
@@ -1539,7 +1567,7 @@ lbve_status build_entries(lbve_pool *P) {
         lbve_pool::FvGroup grp{tx, (int)slot, 0, 0, 0, 0};
         int fv_first = 0;
         for (size_t m = 0; m < n; ++m) {
-            const lbve_ctx *c = P->members[m];
+            const lbve_ctx *c = P->batch[m];
             int lbe = 0, fve = 0;
             P->kt->batch_tiles(c->d, c->lb_tx, c->fv_tx, &lbe, &fve);
             if (fve != tx) continue;
@@ -1571,7 +1599,7 @@ lbve_status build_entries(lbve_pool *P) {
         cl.n = 0;
         int first = 0;
         for (size_t m = 0; m < n; ++m) {
-            const lbve_ctx *c = P->members[m];
+            const lbve_ctx *c = P->batch[m];
             if ((int)(c->t & 1) != par) continue;
             DevState d = c->d;
             d.step = (unsigned)c->t;
@@ -1589,7 +1617,7 @@ lbve_status build_entries(lbve_pool *P) {
     const size_t pb = P->kt->part_entry_bytes;
     std::vector<unsigned char> phost;
     int np_ = 0;
-    for (lbve_ctx *c : P->members) {
+    for (lbve_ctx *c : P->batch) {
         if (c->nparts <= 0) continue;
         phost.resize(pb * (size_t)(np_ + 1));
         const PartScratch ps = part_scratch(c);
@@ -1605,7 +1633,7 @@ lbve_status build_entries(lbve_pool *P) {
     P->n_pentries = np_;
     if (np_) PCK(cudaMemcpyAsync(P->pentries, phost.data(), pb * (size_t)np_, cudaMemcpyHostToDevice, P->stream),
                  "upload particle entries");
-    PCK(cudaMemsetAsync(P->dstep, 0, sizeof(unsigned), P->stream), "step counter reset");
+    PCK(cudaMemsetAsync(P->dstep, 0, 2 * sizeof(unsigned), P->stream), "step counter reset");
     PCK(cudaStreamSynchronize(P->stream), "entries sync");
     if (!P->grid_lb) P->grid_lb = P->kt->batched_grid(0);
     P->dirty = false;
@@ -1625,11 +1653,25 @@ lbve_status ensure_side_streams(lbve_pool *P) {
     return LBVE_OK;
 }
 
+// Side streams [first, first + count) wait for the pool stream; the pool stream for them.
+lbve_status side_fork(lbve_pool *P, int first, int count) {
+    PCK(cudaEventRecord(P->ev_fork, P->stream), "fork");
+    for (int j = first; j < first + count; ++j) PCK(cudaStreamWaitEvent(P->side[j], P->ev_fork, 0), "fork wait");
+    return LBVE_OK;
+}
+lbve_status side_join(lbve_pool *P, int first, int count) {
+    for (int j = first; j < first + count; ++j) {
+        PCK(cudaEventRecord(P->ev_join[j], P->side[j]), "join");
+        PCK(cudaStreamWaitEvent(P->stream, P->ev_join[j], 0), "join wait");
+    }
+    return LBVE_OK;
+}
+
 // Run body(member, stream) for every listed member: on the pool stream when there is one
-// member, else spread over the side streams between a fork and a join on the pool stream.
+// member, else spread over the side streams from `first` on between a fork and a join.
 template <class Body>
-lbve_status fan_out(lbve_pool *P, const std::vector<lbve_ctx *> &list, Body &&body) {
-    const int ns = std::min<int>(lbve_pool::kSide, (int)list.size());
+lbve_status fan_out(lbve_pool *P, const std::vector<lbve_ctx *> &list, int first, Body &&body) {
+    const int ns = std::min<int>(lbve_pool::kSide - first, (int)list.size());
     if (ns <= 1 || !P->side_ready) {
         for (lbve_ctx *c : list) {
             lbve_status s = body(c, P->stream);
@@ -1637,40 +1679,63 @@ lbve_status fan_out(lbve_pool *P, const std::vector<lbve_ctx *> &list, Body &&bo
         }
         return LBVE_OK;
     }
-    PCK(cudaEventRecord(P->ev_fork, P->stream), "fork");
-    for (int j = 0; j < ns; ++j) PCK(cudaStreamWaitEvent(P->side[j], P->ev_fork, 0), "fork wait");
-    for (size_t i = 0; i < list.size(); ++i) {
-        lbve_status s = body(list[i], P->side[i % ns]);
-        if (s != LBVE_OK) return s;
-    }
-    for (int j = 0; j < ns; ++j) {
-        PCK(cudaEventRecord(P->ev_join[j], P->side[j]), "join");
-        PCK(cudaStreamWaitEvent(P->stream, P->ev_join[j], 0), "join wait");
+    lbve_status s = side_fork(P, first, ns);
+    for (size_t i = 0; i < list.size() && s == LBVE_OK; ++i) s = body(list[i], P->side[first + (int)(i % ns)]);
+    if (s != LBVE_OK) return s;
+    return side_join(P, first, ns);
+}
+
+lbve_status member_bodies(lbve_pool *P, lbve_ctx *c, const DevState &d, int parity, cudaStream_t st) {
+    PCK(c->kt->momentum_exchange(d, parity, c->links, c->seg_begin, c->seg_count, c->nbody, c->max_seg_len, c->contrib,
+                                 st),
+        "pool momentum exchange");
+    if (!phase_sums(c)) PCK(body_sums(c, d.parts, st), "pool body sums");
+    return LBVE_OK;
+}
+
+// A member's whole call on a stream of its own (members do not depend on one another).
+lbve_status enqueue_own(lbve_pool *P, lbve_ctx *c, int nsteps, cudaStream_t st) {
+    DevState d = c->d;
+    d.in_pool = 1;
+    d.dstep = P->dstep + 1;
+    for (int k = 0; k < nsteps; ++k) {
+        const int parity = (int)((c->t + k) & 1);
+        // at the call, *dstep is the number of steps since the build (now and in replays)
+        d.step = (unsigned)(c->t - P->steps_since_build + k);
+        if (c->nbody > 0 && (c->nparts > 0 || k + 1 == nsteps)) {
+            lbve_status s = member_bodies(P, c, d, parity, st);
+            if (s != LBVE_OK) return s;
+        }
+        PCK(c->kt->lb(d, parity, st), "pool lb");
+        PCK(c->kt->fv(d, st), "pool fv");
+        d.cur ^= 1;
+        if (c->nparts > 0) PCK(c->kt->particle_phase(d, parity ^ 1, part_scratch(c), st), "pool particle phase");
     }
     return LBVE_OK;
 }
 
-// Enqueue nsteps steps of every member on the pool stream (graph-capturable).
+// Enqueue nsteps steps of every member on the pool stream (graph-capturable): the large
+// members' calls on the lower half of the side streams, the others together by the batched
+// kernels, their momentum exchange on the upper half.
 lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
-    const int n = (int)P->members.size();
-    std::vector<lbve_ctx *> with_bodies, with_parts;
-    for (lbve_ctx *c : P->members)
-        if (c->nparts > 0) with_parts.push_back(c);
-    for (int k = 0; k < nsteps; ++k) {
+    const int n_own = std::min<int>(P->batch.empty() ? lbve_pool::kSide : lbve_pool::kSide / 2, (int)P->own.size());
+    if (n_own > 0) {
+        lbve_status s = side_fork(P, 0, n_own);
+        for (size_t i = 0; i < P->own.size() && s == LBVE_OK; ++i)
+            s = enqueue_own(P, P->own[i], nsteps, P->side[i % (size_t)n_own]);
+        if (s != LBVE_OK) return s;
+    }
+    std::vector<lbve_ctx *> with_bodies;
+    for (int k = 0; k < nsteps && !P->batch.empty(); ++k) {
         const int kk = q + k;  // steps since the entries were built (they encode that state)
         // members with wall classes only: the forces of the call's last step (see lbve_step)
         with_bodies.clear();
-        for (lbve_ctx *c : P->members)
+        for (lbve_ctx *c : P->batch)
             if (c->nbody > 0 && (c->nparts > 0 || k + 1 == nsteps)) with_bodies.push_back(c);
-        lbve_status s = fan_out(P, with_bodies, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
+        lbve_status s = fan_out(P, with_bodies, lbve_pool::kSide / 2, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
             DevState d = c->d;  // the member's state at the start of this call
             if (k & 1) d.cur ^= 1;
-            const int parity = (int)((c->t + k) & 1);
-            PCK(c->kt->momentum_exchange(d, parity, c->links, c->seg_begin, c->seg_count, c->nbody, c->max_seg_len,
-                                         c->contrib, st),
-                "pool momentum exchange");
-            if (!phase_sums(c)) PCK(body_sums(c, d.parts, st), "pool body sums");
-            return LBVE_OK;
+            return member_bodies(P, c, d, (int)((c->t + k) & 1), st);
         });
         if (s != LBVE_OK) return s;
         for (int par = 0; par < 2; ++par) {  // the group of build parity par is at parity (par + kk) & 1
@@ -1680,16 +1745,21 @@ lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
                                   cl.n, cl.total, kk, P->grid_lb, P->dstep, (par + kk) & 1, P->stream),
                 "batched lb");
         }
-        k_step_count<<<1, 1, 0, P->stream>>>(P->dstep);
+        k_step_count<<<1, 1, 0, P->stream>>>(P->dstep, 1u);
         PCK(cudaGetLastError(), "step counter");
         for (const lbve_pool::FvGroup &grp : P->fv_groups)
             PCK(P->kt->fv_batched((const unsigned char *)P->entries[0] + (size_t)grp.start * P->kt->batch_entry_bytes,
                                   grp.n, grp.total, kk, grp.grid, grp.tx, grp.var, P->stream),
                 "batched fv");
-        // particle update, fill/drain and links of every member with particles: one block
-        // per member in one launch
-        if (!with_parts.empty())
-            PCK(P->kt->particle_phase_batched(P->pentries, P->n_pentries, kk, P->stream), "pool particle phase");
+        // particle update, fill/drain and links of every batched member with particles: one
+        // cluster per member in one launch
+        PCK(P->kt->particle_phase_batched(P->pentries, P->n_pentries, kk, P->stream), "pool particle phase");
+    }
+    if (n_own > 0) {
+        lbve_status s = side_join(P, 0, n_own);
+        if (s != LBVE_OK) return s;
+        k_step_count<<<1, 1, 0, P->stream>>>(P->dstep + 1, (unsigned)nsteps);
+        PCK(cudaGetLastError(), "step counter");
     }
     return LBVE_OK;
 }
@@ -1709,7 +1779,7 @@ lbve_status lbve_pool_create(int pdf_prec, size_t budget_bytes, void *cuda_strea
     P->budget = budget_bytes;
     P->stream = (cudaStream_t)cuda_stream;
     P->kt = kt;
-    if (cudaMalloc(&P->dstep, sizeof(unsigned)) != cudaSuccess) {
+    if (cudaMalloc(&P->dstep, 2 * sizeof(unsigned)) != cudaSuccess) {
         cudaGetLastError();
         delete P;
         return LBVE_ENOMEM;
@@ -1796,9 +1866,7 @@ lbve_status lbve_pool_step(lbve_pool *P, int nsteps) {
         if (s != LBVE_OK) return s;
     }
     const int q = (int)(P->steps_since_build & 1);
-    // the legacy default stream cannot be captured: launch directly there
-    const bool graphs = P->use_graphs && (uintptr_t)P->stream > 1;
-    if (graphs) {
+    if (pool_graphs(P)) {
         if (!P->graph[q] || P->graph_steps[q] != nsteps) {
             if (P->graph[q]) cudaGraphExecDestroy(P->graph[q]);
             P->graph[q] = nullptr;
@@ -1829,19 +1897,31 @@ lbve_status lbve_pool_residuals(lbve_pool *P, double *out) {
     if (!P || !out) return P ? pfail(P, LBVE_EINVAL, "out is NULL") : LBVE_EINVAL;
     const size_t n = P->members.size();
     if (n == 0) return LBVE_OK;
-    for (lbve_ctx *c : P->members) {
-        lbve_status s = residual_enqueue(c);
-        if (s != LBVE_OK) return pfail(P, s, c->err);
+    {
+        lbve_status s = ensure_side_streams(P);
+        if (s != LBVE_OK) return s;
     }
-    std::vector<double> h(2 * 1024);
-    for (size_t m = 0; m < n; ++m) {
-        lbve_ctx *c = P->members[m];
-        PCK(cudaMemcpyAsync(h.data(), c->res_partial, sizeof(double) * 2 * residual_blocks(c), cudaMemcpyDeviceToHost,
-                            P->stream),
-            "residual copy");
-        PCK(cudaStreamSynchronize(P->stream), "residual sync");
-        residual_finish(c, h.data(), out + 2 * m);
+    // the members' partial sums side by side into one buffer, one copy, one wait
+    std::vector<size_t> at(n + 1, 0);
+    for (size_t m = 0; m < n; ++m) at[m + 1] = at[m] + 2 * (size_t)residual_blocks(P->members[m]);
+    if (at[n] > P->res_cap) {
+        if (P->res_dev) cudaFree(P->res_dev);
+        P->res_dev = nullptr;
+        P->res_cap = 0;
+        PCK(cudaMalloc(&P->res_dev, sizeof(double) * at[n]), "residual staging");
+        P->res_cap = at[n];
     }
+    size_t next = 0;
+    lbve_status s = fan_out(P, P->members, 0, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
+        lbve_status r = residual_enqueue(c, P->res_dev + at[next++], st);
+        return r == LBVE_OK ? r : pfail(P, r, c->err);
+    });
+    if (s != LBVE_OK) return s;
+    std::vector<double> h(at[n]);
+    PCK(cudaMemcpyAsync(h.data(), P->res_dev, sizeof(double) * at[n], cudaMemcpyDeviceToHost, P->stream),
+        "residual copy");
+    PCK(cudaStreamSynchronize(P->stream), "residual sync");
+    for (size_t m = 0; m < n; ++m) residual_finish(P->members[m], h.data() + at[m], out + 2 * m);
     return LBVE_OK;
 }
 
@@ -1851,6 +1931,7 @@ lbve_status lbve_pool_set_graphs(lbve_pool *P, int enable) {
     if (!P) return LBVE_EINVAL;
     cudaStreamSynchronize(P->stream);
     P->use_graphs = enable != 0;
+    P->dirty = true;  // which members the batched kernels take depends on it
     drop_graphs(P);
     return LBVE_OK;
 }

@@ -67,6 +67,7 @@ struct KArgs {
     const uint32_t *mask;
     const PartDev *parts;
     unsigned step;  // index of the step being performed (rounding keys of keyed stores)
+    const unsigned *dstep;  // added to it (nullptr: nothing)
     unsigned *bad;  // instability flag (mapped host word) or nullptr
     int zlo, zhi;   // planes the step kernels compute
     unsigned key_base;  // added to the cell index in rounding keys (a z-slab: its global offset)
@@ -150,7 +151,8 @@ __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, un
         // 16-bit storage: the pairs (i, -i) round together (stochastically, see Store); a
         // bounce from a resting wall stores the very bits of the normal store (one of the
         // two copies is never read), a moving-wall bounce rounds its own value
-        const uint32_t h = fmix32((r + a.key_base) ^ (a.step * 0x9E3779B9u));
+        const unsigned step = a.dstep ? a.step + *a.dstep : a.step;
+        const uint32_t h = fmix32((r + a.key_base) ^ (step * 0x9E3779B9u));
         const uint32_t d0 = Store<S>::round2(fs[0], fs[0], sc, pair_bits(h, 0));
         Store<S>::store16(a.fq[0] + r, d0);
         if (!__any_sync(__activemask(), moving)) {

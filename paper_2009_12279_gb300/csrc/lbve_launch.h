@@ -105,6 +105,11 @@ struct DevState {
     // launch_step); 0: plain launches (pools, phases, captured streams)
     int pdl = 0;
     int sms = 0;  // SMs of the device (0: asked for when needed)
+    // a member of a pool stepped by kernels of its own beside the others': the stress kernel
+    // of most cells per SM and time, whatever the grid's size, and rounding keys counted from
+    // *dstep on (the launches are replayed from a graph)
+    int in_pool = 0;
+    const unsigned *dstep = nullptr;
 };
 
 #ifdef __CUDACC__

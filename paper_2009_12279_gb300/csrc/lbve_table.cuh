@@ -77,6 +77,7 @@ struct Launch {
         a.mask = d.mask;
         a.parts = d.parts;
         a.step = d.step;
+        a.dstep = d.dstep;
         a.bad = d.bad;
         a.zlo = d.zlo;
         a.zhi = d.zhi > 0 ? d.zhi : d.g.nz;
@@ -295,13 +296,16 @@ struct Launch {
         if constexpr (!Store<S>::shifted) {
             return false;
         } else {
-            auto al = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
-            if (!d.auto_kernels || fv_variant(d) || d.g.nx % 4 != 0) return false;
+            if (!d.auto_kernels || !fv_pair_shape(d)) return false;
             // schedule AUTO: grids of 2^21 cells and more (measured on GB300: 12 % faster at
             // 128^3, slower below about 10^6 cells, where its 512-cell columns leave SMs idle)
-            if (d.auto_kernels == 1 && d.g.n < (1LL << 21)) return false;
-            return al(d.tau[0]) && al(d.tau[1]) && al(d.u[0]) && al(d.u[1]) && al(d.mask);
+            return d.auto_kernels != 1 || d.g.n >= (1LL << 21);
         }
+    }
+    static bool fv_pair_shape(const DevState &d) {
+        auto al = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
+        return Store<S>::shifted && !fv_variant(d) && d.g.nx % 4 == 0 && al(d.tau[0]) && al(d.tau[1]) && al(d.u[0]) &&
+               al(d.u[1]) && al(d.mask);
     }
     static int fv_pair_used(const DevState &d) { return fv_pair_ok(d) ? 1 : 0; }
     // z-planes per block of the two-cell stress kernel (~16 waves of 2 resident blocks)
@@ -328,6 +332,18 @@ struct Launch {
         }
     }
     static cudaError_t fv(const DevState &d, cudaStream_t s) {
+        if constexpr (Store<S>::shifted) {
+            if (d.in_pool) {
+                // beside other members the chip is full: the kernels that take least SM time
+                // per cell (256^3, FP32: two-cell 15 ps, tiled 17, per-cell 31), rows of half a
+                // column and more
+                DevState q = d;
+                q.fv_zchunk = fv_zchunk_batched(d);
+                if (d.g.nx >= 64 && fv_pair_shape(d)) return fv_pair(q, s);
+                if (d.g.nx >= 32) return fv_variant(d) ? fv_var<true>(q, s) : fv_var<false>(q, s);
+                return fv_cells(d, s);
+            }
+        }
         if (fv_cells_ok(d)) return fv_cells(d, s);
         if (fv_pair_ok(d)) return fv_pair(d, s);
         if constexpr (Store<S>::shifted) return fv_variant(d) ? fv_var<true>(d, s) : fv_var<false>(d, s);

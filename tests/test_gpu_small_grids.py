@@ -60,3 +60,52 @@ def test_per_cell_stress_equals_tiled_bitwise(precision, shape, periodic, kw):
     b = _run(shape, periodic, precision, lbve.SCHED_SPLIT, (1, 4, 2), **kw)
     for name, x, y in zip(("pdfs", "rho", "u", "tau", "body forces"), a, b):
         assert np.array_equal(x, y), name
+
+
+@pytest.mark.parametrize("precision", ["bf16", "f32"])
+def test_pool_members_of_both_kinds_equal_alone(precision):
+    """70 members: the large ones step by kernels of their own, the small ones by the batched
+    kernels; in a pool of 3 every member has its own.  Calls of 1, 4 and 4 steps (graphs of
+    both parities, one replayed).  Fields and PDFs are those of the same solves alone."""
+    import torch
+
+    from paper_2009_12279_gb300 import Pool, Solver, workloads
+
+    shapes = [(64, 40, 32), (48, 48, 32), (16, 12, 10)] + [(9 + k % 7, 8, 7) for k in range(67)]
+
+    def solver(k, stream):
+        shape = shapes[k]
+        fl = workloads.channel_flags(shape, 1)
+        fl |= workloads.random_obstacles(shape, 0.03, k).astype(fl.dtype)
+        fl[2, 3, 4] = 2  # a tracked wall cell
+        s = Solver(shape, precision=precision, stream=stream, periodic=(1, 0, 1), lambda_p=150.0, beta=0.4,
+                   body_force=(1e-5, 0.0, 0.0), giesekus_alpha=0.2 if k == 1 else 0.0)
+        s.set_geometry(fl, [(0.01, 0.0, 0.0)])
+        s.init_fields(u=workloads.random_velocity(shape, 1e-3, k) * (fl == 0))
+        return s
+
+    for members in (70, 3):
+        stream = torch.cuda.Stream()
+        pool = Pool(precision, stream=stream.cuda_stream)
+        mine = [solver(k, stream.cuda_stream) for k in range(members)]
+        for s in mine:
+            pool.admit(s)
+        for n in (1, 4, 4):
+            pool.step(n)
+        res = pool.residuals()
+        for k in list(range(4)) + [members - 1]:
+            if k >= members:
+                continue
+            alone = solver(k, 0)
+            for n in (1, 4, 4):
+                alone.step(n)
+            assert np.array_equal(alone.read_pdfs(), mine[k].read_pdfs()), (members, k)
+            for a, b in zip(alone.read_fields(), mine[k].read_fields()):
+                assert np.array_equal(a, b), (members, k)
+            assert np.array_equal(alone.body_forces(), mine[k].body_forces()), (members, k)
+            assert alone.residual() == tuple(res[k]), (members, k)
+            alone.close()
+        for s in mine:
+            pool.remove(s)
+            s.close()
+        pool.close()
