@@ -82,12 +82,13 @@ typedef enum { LBVE_F64 = 0, LBVE_F32 = 1, LBVE_F16_SHIFTED = 2, LBVE_BF16_SHIFT
 
 /* Kernel schedule: two kernels per step (LB, then FV), or one fused kernel per step.
  * SPLIT: the per-cell stream-collide (the LB half, Eqs. (lb), (guo), (force), (ubb)) and
- * the tiled stress update (FP64: the per-cell stress update).  PIPELINED: the split schedule with the row-pipelined
- * stream-collide and the two-cell stress update wherever the grid allows them (see
- * lbve_stream_collide_kernel, lbve_stress_kernel).  AUTO: PIPELINED for large grids (the
- * row pipeline from 2^22 cells in FP32 and 16-bit storage, the two-cell stress update
- * from 2^21, where they were measured faster on GB300), SPLIT below, with a per-cell
- * stress update below 3 * 2^18 cells.  All three give bitwise the same results. */
+ * the tiled stress update (FP64: the per-cell stress update).  PIPELINED: the split
+ * schedule with the row-pipelined stream-collide and the two-cell stress update wherever
+ * the grid allows them (see lbve_stream_collide_kernel, lbve_stress_kernel).  AUTO:
+ * PIPELINED for large grids (the row pipeline from 2^22 cells in FP32 and 16-bit storage
+ * where rows of this length fill an SM, the two-cell stress update from 2^21, where they
+ * were measured faster on GB300), SPLIT below, with a per-cell stress update below
+ * 3 * 2^18 cells.  All three give bitwise the same results. */
 #define LBVE_SCHED_AUTO 0
 #define LBVE_SCHED_SPLIT 1
 #define LBVE_SCHED_FUSED 2
@@ -261,7 +262,8 @@ int lbve_is_unstable(const lbve_ctx *ctx);
  * producer warp moves each row's 19 PDF rows (AA layout of the step's parity), its mask
  * row and the stress rows its polymer force reads (Eq. (force): the rows y -+ 1 and
  * z -+ 1) into shared memory with bulk asynchronous copies completing on mbarriers.  It
- * is taken with schedule PIPELINED (AUTO: from 2^22 cells, FP32 and 16-bit storage) when
+ * is taken with schedule PIPELINED (AUTO: from 2^22 cells, FP32 and 16-bit storage, for
+ * row lengths of which an SM's shared memory holds 15 / 16 warps' worth) when
  * nx is a multiple of 32 in [64, 512], the PDF, stress and mask arrays are 16-byte
  * aligned (always with the library's own allocations), the layout fits one block's
  * shared memory (FP64: nx up to 384) and the stress law is not FENE-P.  LBVE_LB_CELLS:

@@ -19,16 +19,13 @@
 namespace lbve {
 
 // 128-thread stream-collide blocks with a resident-block floor per SM, i.e. a register
-// cap of 65536 / (128 x floor): without a cap the odd-parity kernel keeps all 37
-// neighbour addresses live and drops to ~10 % occupancy.  Measured at 512^3: FP32 runs
-// fastest at 7 blocks (72 registers; 8 blocks spill more, 9 or more lose); with the
-// stochastically rounded 16-bit stores BF16 at 7 (4.00 ms against 4.03 at 8) and FP16 at
-// 8 (4.03 ms against 4.09 at 7); FP64, bound by its pipe from a few warps on, at 4 (no
-// spills).
-template <class S, int PAR>
+// cap of 65536 / (128 x floor).  FP32 and 16-bit storage take 72 registers (7 blocks, no
+// spills): measured on GB300 at 192^3, us, with 5 / 6 / 7 / 8 / 9 blocks: FP32 293 / 253 /
+// 248 / 257 / 255; BF16 239 / 208 / 198 / 209 / 206; FP16 at 128^3 72 / - / 65 / 70 / 68.
+// FP64, bound by its pipe from a few warps on, takes 128 (4 blocks, no spills).
+template <class S>
 constexpr int lb_min_blocks() {
-    if (sizeof(S) == 8) return 4;
-    return (sizeof(S) == 4 || std::is_same<S, __nv_bfloat16>::value) ? 7 : 8;
+    return sizeof(S) == 8 ? 4 : 7;
 }
 // 256-thread stress blocks, 3 resident per SM (80 registers: no spills at 4)
 #ifndef LBVE_FV_MIN_BLOCKS
@@ -308,7 +305,7 @@ __device__ __forceinline__ void lb_cell_at(const KArgs<S> &a, int x, int y, int 
 
 // FENE: the stress arrays hold FENE-P conformation tensors (see polymer_force_core_fene)
 template <class S, int PAR, bool FENE, bool LIN>
-__global__ void __launch_bounds__(128, lb_min_blocks<S, PAR>()) k_lb(KArgs<S> a) {
+__global__ void __launch_bounds__(128, lb_min_blocks<S>()) k_lb(KArgs<S> a) {
     step_wait();
     int x, y, z;
     if (!cell_of_thread<S, LIN>(a, x, y, z)) return;
@@ -343,9 +340,11 @@ __device__ __forceinline__ void fv_cell_at(const KArgs<S> &a, int x, int y, int 
 // Per-cell stress update, for grids whose z-marching columns would not fill the chip (and
 // all FP64 ones).  Bound by latency there (one round of loads, then the arithmetic), so it
 // is split as finely as it goes: one cell per thread, 128-thread blocks, the neighbours'
-// values through L1 (a 32^3 grid: 256 blocks in 7.7 us, where 8 columns took 20.3).
+// values through L1 (a 32^3 grid: 256 blocks in 7.7 us, where 8 columns took 20.3).  72
+// registers: FENE-P 100 x 84 x 60 at 5 / 6 / 7 / 8 blocks per SM 20.4 / 19.2 / 18.7 / 18.2 us,
+// Oldroyd-B 15.7 / 14.2 / 14.1 / 14.7.
 template <class S, bool VAR, bool LIN>
-__global__ void __launch_bounds__(128, 5) k_fv_cells(KArgs<S> a) {
+__global__ void __launch_bounds__(128, sizeof(S) == 8 ? 5 : 7) k_fv_cells(KArgs<S> a) {
     step_wait();
     int x, y, z;
     if (!cell_of_thread<S, LIN>(a, x, y, z)) return;

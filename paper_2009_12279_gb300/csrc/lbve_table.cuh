@@ -113,19 +113,29 @@ struct Launch {
     static bool rows_ok(const DevState &d) {
         auto al = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
         if (d.ph.fene || d.g.nx % 32 != 0 || d.g.nx < 64 || d.g.nx > LR_MAX_NX) return false;
-        // schedule AUTO: grids of 2^22 cells and more in the FP32 / 16-bit modes (measured
-        // on GB300: at 128^3 the two stream-collides take the same time, below it the
-        // per-cell kernel is faster, the row pipeline's per-block fill not being hidden;
-        // the FP64 parity mode keeps the per-cell kernel)
+        // schedule AUTO: grids of 2^22 cells and more (FP64, the parity mode: never) ...
         if (d.auto_kernels == 1 && (d.g.n < (1LL << 22) || !Store<S>::shifted)) return false;
         if (!al(d.f) || !al(d.tau[0]) || !al(d.tau[1]) || !al(d.mask) || !al(d.u[0]) || !al(d.u[1])) return false;
-        int dev = 0, optin = 0;
+        int dev = 0, optin = 0, persm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return false;
         if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return false;
-        return rows_smem(d.g.nx) <= (size_t)optin;
+        const size_t sm = rows_smem(d.g.nx);
+        if (sm > (size_t)optin) return false;
+        if (d.auto_kernels != 1) return true;
+        // ... whose rows fill an SM: the blocks that fit its shared memory have nx / 32
+        // consumer warps each, and below 15 (FP32; 16 with 16-bit storage) of them the per-cell
+        // kernel, which has 28, is faster.  Measured on GB300, 6 M cells, row pipeline against
+        // per-cell, us: FP32 192-wide (12 warps) 238 / 212, 224 (14) 216 / 212, 256 (16) 203 /
+        // 212, 320 (10) 257 / 212, 512 (16) 207 / 214, and 256^3 542 / 621; BF16 192 (12) 229 /
+        // 174, 288 (9) 276 / 182, 512^2 x 64 (16) 509 / 496.
+        if (cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) return false;
+        const int warps = (int)((size_t)persm / (sm + 1024)) * (d.g.nx / 32);
+        return d.g.nx >= 128 && warps >= (sizeof(S) == 2 ? 16 : 15);
     }
-    // rows per strip: enough strips for ~16 waves of resident blocks (d.lb_rows_yc > 0:
-    // that many), at least 8 rows
+    // rows per strip (d.lb_rows_yc > 0: that many): enough strips for ~16 waves of resident
+    // blocks, at least 8 rows; 16-bit storage 8 waves and 16 rows (a strip costs about a row
+    // more than it has: BF16 512^2 x 64 509 -> 474 us, 256^3 512 -> 503; FP32, where memory
+    // is the bound, loses 1 %)
     static RowsWork rows_work(const DevState &d, size_t smem) {
         const int ny = d.g.ny, nzc = zcount(d);
         int yc = d.lb_rows_yc;
@@ -137,11 +147,11 @@ struct Launch {
             }
             long long per_sm = smpb > 0 ? (long long)smpb / (long long)(smem + 1024) : 1;
             if (per_sm < 1) per_sm = 1;
-            const long long want = 16LL * sms * per_sm;
+            const long long want = (sizeof(S) == 2 ? 8LL : 16LL) * sms * per_sm;
             long long strips = (want + nzc - 1) / nzc;
             if (strips < 1) strips = 1;
             yc = (int)((ny + strips - 1) / strips);
-            if (yc < 8) yc = 8;
+            if (yc < (sizeof(S) == 2 ? 16 : 8)) yc = sizeof(S) == 2 ? 16 : 8;
         }
         if (yc > ny) yc = ny;
         RowsWork w;
