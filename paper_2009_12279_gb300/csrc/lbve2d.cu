@@ -414,10 +414,11 @@ struct lbve2d_ctx {
     void *f[2] = {nullptr, nullptr}, *tau[2] = {nullptr, nullptr}, *u = nullptr, *ub = nullptr, *force = nullptr;
     uint8_t *flag = nullptr;
     double *stage = nullptr;  // FP64 staging, 10 n doubles
+    // set up by the first call that takes several steps in one launch:
     unsigned *bar = nullptr;    // device word of the grid barrier
     unsigned *stuck = nullptr;  // mapped host word: 2 once a barrier's bounded wait gave up
     unsigned *stuck_dev = nullptr;
-    int resident = 0;           // tiles the device holds at once
+    int resident = -1;          // tiles the device holds at once (-1: not asked yet)
     Phys2<double> ph;
     std::string err;
 };
@@ -489,6 +490,23 @@ const char *const kStuck = "the blocks of a multi-step launch gave up waiting fo
 dim3 block2d() { return dim3(64, 2); }
 dim3 grid2d(const lbve2d_ctx *c) { return dim3((unsigned)((c->p.nx + 63) / 64), (unsigned)((c->p.ny + 1) / 2)); }
 
+cudaError_t multi_setup(lbve2d_ctx *c) {
+    if (c->stuck) return cudaSuccess;
+    cudaError_t e = c->bar ? cudaSuccess : cudaMalloc((void **)&c->bar, sizeof(unsigned));
+    if (e != cudaSuccess) return e;
+    unsigned *w = nullptr;
+    e = cudaHostAlloc((void **)&w, sizeof(unsigned), cudaHostAllocMapped);
+    if (e != cudaSuccess) return e;
+    *w = 0u;
+    e = cudaHostGetDevicePointer((void **)&c->stuck_dev, w, 0);
+    if (e != cudaSuccess) {
+        cudaFreeHost(w);
+        return e;
+    }
+    c->stuck = w;
+    return cudaSuccess;
+}
+
 dim3 tiles2d(const lbve2d_ctx *c) {
     return dim3((unsigned)((c->p.nx + T2X - 1) / T2X), (unsigned)((c->p.ny + T2Y - 1) / T2Y));
 }
@@ -500,10 +518,13 @@ dim3 tiles2d(const lbve2d_ctx *c) {
 template <class R, bool SH>
 cudaError_t step_impl(lbve2d_ctx *c, int nsteps) {
     const dim3 g = tiles2d(c);
+    if (c->resident < 0) c->resident = lbve::resident_blocks(k2_steps<R, SH>, T2THREADS, 0);
     const bool fits = (long long)g.x * g.y <= c->resident;
     if (nsteps > 1 && fits && !lbve::capturing(c->stream)) {
+        cudaError_t e = multi_setup(c);
+        if (e != cudaSuccess) return e;
         Args2<R> a = args2<R>(c);
-        cudaError_t e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
+        e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
         if (e != cudaSuccess) return e;
         void *args[] = {&a, &nsteps, &c->bar, &c->stuck_dev};
         e = cudaLaunchCooperativeKernel((const void *)k2_steps<R, SH>, g, dim3(T2THREADS), args, 0, c->stream);
@@ -597,12 +618,6 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
     if (e == cudaSuccess) e = cudaMalloc(&c->ub, 2 * n * c->rb);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->flag, n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&c->stage, 15 * n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->bar, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->stuck, sizeof(unsigned), cudaHostAllocMapped);
-    if (e == cudaSuccess) {
-        *c->stuck = 0u;
-        e = cudaHostGetDevicePointer((void **)&c->stuck_dev, c->stuck, 0);
-    }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->flag, 0, n, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ub, 0, 2 * n * c->rb, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->u, 0, 2 * n * c->rb, c->stream);
@@ -614,8 +629,6 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
         lbve2d_destroy(c);
         return e == cudaErrorMemoryAllocation ? LBVE_ENOMEM : LBVE_ECUDA;
     }
-    c->resident = c->rb == 8 ? lbve::resident_blocks(k2_steps<double, false>, T2THREADS, 0)
-                             : lbve::resident_blocks(k2_steps<float, true>, T2THREADS, 0);
     lbve_status s = lbve2d_init_fields(c, nullptr, nullptr, nullptr);
     if (s != LBVE_OK) {
         g_err2 = c->err;
@@ -693,7 +706,7 @@ lbve_status lbve2d_init_fields(lbve2d_ctx *c, const double *rho, const double *u
     }
     CK2(cudaGetLastError(), "init kernel");
     CK2(cudaStreamSynchronize(c->stream), "init sync");
-    *(volatile unsigned *)c->stuck = 0u;
+    if (c->stuck) *(volatile unsigned *)c->stuck = 0u;
     c->t = 0;
     return LBVE_OK;
 }
