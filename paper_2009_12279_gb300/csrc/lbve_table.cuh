@@ -318,12 +318,29 @@ struct Launch {
                al(d.u[1]) && al(d.mask);
     }
     static int fv_pair_used(const DevState &d) { return fv_pair_ok(d) ? 1 : 0; }
-    // z-planes per block of the two-cell stress kernel (~16 waves of 2 resident blocks)
+    // z-planes per block of the two-cell stress kernel: ~16 waves of 2 resident blocks; where
+    // 16-plane chunks make less than 8, the chunk of least predicted time (see fv_zchunk): a
+    // plane takes 2.1 us with two blocks on an SM and 1.3 with one, and a block 1.5 planes
+    // more than it updates.  FP32, event-timed: 128^3 43.2 -> 41.4 us, 192 x 160 x 96 64.1 ->
+    // 53.5 (chunks of 20: 300 blocks on 304 places), 256^3 257 -> 248.
     static int fv_pair_zchunk(const DevState &d) {
         const int nz = zcount(d);
         if (d.fv_zchunk > 0) return d.fv_zchunk < nz ? d.fv_zchunk : nz;
         const long long tiles = (long long)((d.g.nx + FP_TX - 1) / FP_TX) * ((d.g.ny + FP_TY - 1) / FP_TY);
-        return march_zchunk(tiles, nz, 2LL * sm_count());
+        const long long sms = d.sms > 0 ? d.sms : sm_count(), slots = 2 * sms;
+        int best = march_zchunk(tiles, nz, slots);
+        if (best > 16 || tiles * ((nz + 15) / 16) >= 8 * slots) return best;
+        double least = 0.0;
+        for (int chunks = 1; chunks <= (nz + 7) / 8; ++chunks) {
+            const int zc = (nz + chunks - 1) / chunks;
+            const long long blocks = tiles * ((nz + zc - 1) / zc), rest = blocks % slots;
+            const double t = (zc + 1.5) * (2.1 * (double)(blocks / slots) + (rest == 0 ? 0.0 : rest <= sms ? 1.3 : 2.1));
+            if (chunks == 1 || t < least) {
+                least = t;
+                best = zc;
+            }
+        }
+        return best;
     }
     static cudaError_t fv_pair(const DevState &d, cudaStream_t s) {
         if constexpr (!Store<S>::shifted) {
