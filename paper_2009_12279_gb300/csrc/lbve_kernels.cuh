@@ -129,6 +129,18 @@ __device__ __forceinline__ R moving_wall_term(R *const (&u)[3], unsigned nb, int
     const R w = i < 7 ? wgt<R>(1) : wgt<R>(7);
     return mul1(mul1(R(6) * w, rho), cub);
 }
+template <class R>
+__device__ __noinline__ R moving_wall_call(R *u, size_t np, unsigned nb, int i, R rho) {
+    R *const uq[3] = {u, u + np, u + 2 * np};
+    return moving_wall_term<R>(uq, nb, i, rho);
+}
+
+// Step number of the rounding key.
+template <class S>
+__device__ __forceinline__ unsigned step_number(const KArgs<S> &a) {
+    if constexpr (Store<S>::keyed) return a.dstep ? a.step + *a.dstep : a.step;
+    return 0u;
+}
 
 // Store post-collision f*_i with AA addressing; links into solid cells bounce back with
 // the moving-wall term of Eq. (ubb): f_-i(r, t+1) = f*_i(r) - 6 w_i rho c_i . u_b.
@@ -137,18 +149,23 @@ __device__ __forceinline__ R moving_wall_term(R *const (&u)[3], unsigned nb, int
 // step: slot -i of r holds f_i(r + c_i)), or is the one this thread itself read before
 // (odd step: slot i of r + c_i held the bounced population f_-i(r)).  The bounced value
 // is an extra store for the links into solid cells only.
-template <class S, int PAR>
+template <class S, int PAR, bool ROWS>
 __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, unsigned r, uint32_t mask,
-                                           const typename Store<S>::R (&fs)[Q], typename Store<S>::R rho) {
+                                           const typename Store<S>::R (&fs)[Q], typename Store<S>::R rho,
+                                           unsigned step) {
     using R = typename Store<S>::R;
     const size_t np = (size_t)a.g.np;
+    auto wall_term = [&](unsigned nb, int i) -> R {
+        if constexpr (ROWS) return moving_wall_call<R>(a.uq[0], np, nb, i, rho);
+        return moving_wall_term<R>(a.uq, nb, i, rho);
+    };
     const R sc = a.ph.scale;
     const bool moving = mask & MASK_MOVING;  // else every solid neighbour is a resting no-slip wall
     if constexpr (Store<S>::keyed) {
         // 16-bit storage: the pairs (i, -i) round together (stochastically, see Store); a
         // bounce from a resting wall stores the very bits of the normal store (one of the
         // two copies is never read), a moving-wall bounce rounds its own value
-        const unsigned step = a.dstep ? a.step + *a.dstep : a.step;
+        if constexpr (!ROWS) step = step_number(a);
         const uint32_t h = fmix32((r + a.key_base) ^ (step * 0x9E3779B9u));
         const uint32_t d0 = Store<S>::round2(fs[0], fs[0], sc, pair_bits(h, 0));
         Store<S>::store16(a.fq[0] + r, d0);
@@ -180,7 +197,7 @@ __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, un
                 Store<S>::store16(PAR == 0 ? a.fq[copp(j)] + r : a.fq[j] + nb, bits);
                 if (!nb_solid(mask, j)) continue;
                 S *dst = PAR == 0 ? a.fq[j] + nb : a.fq[copp(j)] + r;
-                const R X = moving ? moving_wall_term<R>(a.uq, nb, j, rho) : R(0);
+                const R X = moving ? wall_term(nb, j) : R(0);
                 // a boundary at rest (X exactly zero) bounces the normal store's bits
                 Store<S>::store16(dst, X == R(0) ? bits
                                                  : Store<S>::round2(fs[j] - X, fs[j] - X, sc, pair_bits(h, Q + j)));
@@ -204,7 +221,7 @@ __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, un
         const unsigned nb = cl.idx(cx(i), cy(i), cz(i));
         Store<S>::st(PAR == 0 ? a.fq[copp(i)] + r : a.fq[i] + nb, fs[i], sc);
         if (nb_solid(mask, i)) {
-            const R X = moving ? moving_wall_term<R>(a.uq, nb, i, rho) : R(0);
+            const R X = moving ? wall_term(nb, i) : R(0);
             Store<S>::st(PAR == 0 ? a.fq[i] + nb : a.fq[copp(i)] + r, fs[i] - X, sc);
         }
     }
@@ -212,11 +229,14 @@ __device__ __forceinline__ void store_pdfs(const KArgs<S> &a, const Cell &cl, un
 
 // LB half of the step for one fluid cell, given its own stress tr and an accessor tn for
 // its face neighbours' stress (tau^t): F = g + F^p, moments, u^t written out, TRT
-// collision with forcing, AA streaming with bounce-back.
-template <class S, int PAR, bool FENE = false, class TauNb>
+// collision with forcing, AA streaming with bounce-back.  ROWS: the row pipeline's build.  Its
+// 16 warps on an SM feel the instruction fetch of the rare moving-boundary stores and the
+// step number's load in every cell, so it calls the wall term and passes step_number(a) in
+// (512^3: BF16 3.67 -> 3.54 ms, FP16 3.86 -> 3.64; the per-cell kernels would spill).
+template <class S, int PAR, bool FENE, bool ROWS, class TauNb>
 __device__ __forceinline__ void lb_core_f(const KArgs<S> &a, const Cell &cl, unsigned r, uint32_t mask,
                                           const typename Store<S>::R (&tr)[6], const TauNb &tn,
-                                          typename Store<S>::R (&f)[Q]) {
+                                          typename Store<S>::R (&f)[Q], unsigned step = 0) {
     using R = typename Store<S>::R;
     constexpr bool SH = Store<S>::shifted;
     R Fp[3], F[3], u[3], rho, drho;
@@ -231,7 +251,7 @@ __device__ __forceinline__ void lb_core_f(const KArgs<S> &a, const Cell &cl, uns
 #pragma unroll
     for (int k = 0; k < 3; ++k) a.uq[k][r] = u[k];
     const bool bad = collide<R, SH>(f, rho, drho, u, F, a.ph);
-    store_pdfs<S, PAR>(a, cl, r, mask, f, rho);
+    store_pdfs<S, PAR, ROWS>(a, cl, r, mask, f, rho, step);
     // instability (rho <= 0, |u| at or above the lattice sound speed, or a NaN): a rare
     // store to the host-mapped flag
     if (bad && a.bad != nullptr) *(volatile unsigned *)a.bad = 1u;
@@ -241,7 +261,7 @@ __device__ __forceinline__ void lb_core(const KArgs<S> &a, const Cell &cl, unsig
                                         const typename Store<S>::R (&tr)[6], const TauNb &tn) {
     typename Store<S>::R f[Q];
     load_pdfs<S, PAR>(a, cl, r, f);
-    lb_core_f<S, PAR>(a, cl, r, mask, tr, tn, f);
+    lb_core_f<S, PAR, false, false>(a, cl, r, mask, tr, tn, f);
 }
 
 // Velocity / stress accessors of the face neighbours in global memory
@@ -300,7 +320,7 @@ __device__ __forceinline__ void lb_cell_at(const KArgs<S> &a, int x, int y, int 
         const int k = l >> 1, s = (l & 1) ? -1 : 1;
         return a.tq[c][cl.idx(k == 0 ? s : 0, k == 1 ? s : 0, k == 2 ? s : 0)];
     };
-    lb_core_f<S, PAR, FENE>(a, cl, r, m, tr, tn, f);
+    lb_core_f<S, PAR, FENE, false>(a, cl, r, m, tr, tn, f);
 }
 
 // FENE: the stress arrays hold FENE-P conformation tensors (see polymer_force_core_fene)

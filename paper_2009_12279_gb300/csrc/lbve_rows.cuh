@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(LR_MAX_NX + 32, 1) k_lb_rows(KArgs<S> a, RowsW
 
     // ---------------- consumer threads: cell x of every row ----------------
     const int x = tid;
+    const unsigned step = step_number(a);
     for (int j = 0; j < rows; ++j) {
         const int s = j % NS;
         if (!mbar_wait(&full[s], (unsigned)(j / NS) & 1u)) {
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(LR_MAX_NX + 32, 1) k_lb_rows(KArgs<S> a, RowsW
                     default: return tz_s(s, 0, zface_slot(c))[x];
                 }
             };
-            lb_core_f<S, PAR>(a, cl, r, m, tr, tn, f);
+            lb_core_f<S, PAR, false, true>(a, cl, r, m, tr, tn, f, step);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);

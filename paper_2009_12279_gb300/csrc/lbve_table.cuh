@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 
 #include "lbve_kernels.cuh"
 #include "lbve_particles.cuh"
@@ -132,10 +133,11 @@ struct Launch {
         const int warps = (int)((size_t)persm / (sm + 1024)) * (d.g.nx / 32);
         return d.g.nx >= 128 && warps >= (sizeof(S) == 2 ? 16 : 15);
     }
-    // rows per strip (d.lb_rows_yc > 0: that many): enough strips for ~16 waves of resident
-    // blocks, at least 8 rows; 16-bit storage 8 waves and 16 rows (a strip costs about a row
-    // more than it has: BF16 512^2 x 64 509 -> 474 us, 256^3 512 -> 503; FP32, where memory
-    // is the bound, loses 1 %)
+    // Rows per strip (d.lb_rows_yc > 0: that many).  FP32, where memory is the bound: strips for
+    // ~16 waves of resident blocks, at least 8 rows.  16-bit storage, where an SM's own rate
+    // is: the split of least whole rounds of blocks x (rows + 1.5), 1.5 rows being what a
+    // strip costs to fill and drain, of at most ~32 waves (BF16 512^3, 8 waves 3.93 ms, this
+    // 3.54; 256^3 503 -> 486 us).
     static RowsWork rows_work(const DevState &d, size_t smem) {
         const int ny = d.g.ny, nzc = zcount(d);
         int yc = d.lb_rows_yc;
@@ -147,11 +149,19 @@ struct Launch {
             }
             long long per_sm = smpb > 0 ? (long long)smpb / (long long)(smem + 1024) : 1;
             if (per_sm < 1) per_sm = 1;
-            const long long want = (sizeof(S) == 2 ? 8LL : 16LL) * sms * per_sm;
-            long long strips = (want + nzc - 1) / nzc;
-            if (strips < 1) strips = 1;
-            yc = (int)((ny + strips - 1) / strips);
-            if (yc < (sizeof(S) == 2 ? 16 : 8)) yc = sizeof(S) == 2 ? 16 : 8;
+            const long long places = sms * per_sm;
+            if constexpr (sizeof(S) == 2) {
+                long long best = LLONG_MAX;
+                for (long long n = 1; n <= ny && (n == 1 || n * nzc <= 32 * places); ++n) {
+                    const int rows = (int)((ny + n - 1) / n);
+                    const long long strips = (ny + rows - 1) / rows;
+                    const long long cost = (strips * nzc + places - 1) / places * (2 * rows + 3);
+                    if (cost < best) best = cost, yc = rows;
+                }
+            } else {
+                const long long strips = std::max(1LL, (16 * places + nzc - 1) / nzc);
+                yc = std::max(8, (int)((ny + strips - 1) / strips));
+            }
         }
         if (yc > ny) yc = ny;
         RowsWork w;
