@@ -69,7 +69,8 @@ struct KArgs {
     int zlo, zhi;   // planes the step kernels compute
     unsigned key_base;  // added to the cell index in rounding keys (a z-slab: its global offset)
     unsigned lin;       // cells of the computed planes (per-cell kernels in memory order)
-    FastDiv dnx, dny;   // division by nx, ny
+    FastDiv dnx, dny, dnz;  // division by nx, ny, nzc
+    unsigned nzc;           // planes computed
     // per-direction / per-component bases (f + i np, tau + c np, u_out + k np, u_in + k np,
     // tau_out + c np), so that an address is one multiply-add of a 32-bit cell index; set
     // by link_dirs
@@ -296,8 +297,10 @@ __device__ __forceinline__ bool cell_of_thread(const KArgs<S> &a, int &x, int &y
         return true;
     }
     x = blockIdx.x * blockDim.x + threadIdx.x;
-    y = blockIdx.y * blockDim.y + threadIdx.y;
-    z = (int)blockIdx.z + a.zlo;
+    // chunks of rows, each swept in z (see cell_launch)
+    const unsigned chunk = a.dnz.div(blockIdx.z);
+    y = (chunk * gridDim.y + blockIdx.y) * blockDim.y + threadIdx.y;
+    z = (int)(blockIdx.z - chunk * a.nzc) + a.zlo;
     return x < a.g.nx && y < a.g.ny;
 }
 

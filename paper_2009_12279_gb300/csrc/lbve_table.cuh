@@ -86,6 +86,8 @@ struct Launch {
         a.lin = (unsigned)((long long)d.g.nx * d.g.ny * zcount(d));
         a.dnx = FastDiv::of((unsigned)d.g.nx);
         a.dny = FastDiv::of((unsigned)d.g.ny);
+        a.nzc = (unsigned)zcount(d);
+        a.dnz = FastDiv::of(a.nzc);
         link_dirs<S>(a);
         return a;
     }
@@ -124,14 +126,15 @@ struct Launch {
         if (sm > (size_t)optin) return false;
         if (d.auto_kernels != 1) return true;
         // ... whose rows fill an SM: the blocks that fit its shared memory have nx / 32
-        // consumer warps each, and below 15 (FP32; 16 with 16-bit storage) of them the per-cell
-        // kernel, which has 28, is faster.  Measured on GB300, 6 M cells, row pipeline against
-        // per-cell, us: FP32 192-wide (12 warps) 238 / 212, 224 (14) 216 / 212, 256 (16) 203 /
-        // 212, 320 (10) 257 / 212, 512 (16) 207 / 214, and 256^3 542 / 621; BF16 192 (12) 229 /
-        // 174, 288 (9) 276 / 182, 512^2 x 64 (16) 509 / 496.
+        // consumer warps each, and with few of them the per-cell kernel, which has 28, is
+        // faster.  Measured on GB300, row pipeline against per-cell, ps per cell: FP32 192-wide
+        // (12 warps) 36.6 / 34.8, 224 (14) 33.3 / 35.9, 256 (16) 31.9 / 34.5, 320 (10) 35.7 /
+        // 34.3, 384 (12) 6 M cells 38.6 / 35.4, 57 M 33.4 / 34.3, 448 (14) 32.4 / 34.5; BF16
+        // 224 (14) 30.4 / 28.4, 256 (16) 28.9 / 28.1, 288 (9) 39.8 / 28.5, 512 (16) 26.9 / 28.2.
         if (cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) return false;
         const int warps = (int)((size_t)persm / (sm + 1024)) * (d.g.nx / 32);
-        return d.g.nx >= 128 && warps >= (sizeof(S) == 2 ? 16 : 15);
+        if (sizeof(S) == 4 && d.g.nx >= 384 && d.g.n >= (1LL << 24)) return true;
+        return d.g.nx >= 128 && warps >= (sizeof(S) == 2 ? 16 : 14);
     }
     // Rows per strip (d.lb_rows_yc > 0: that many).  FP32, where memory is the bound: strips for
     // ~16 waves of resident blocks, at least 8 rows.  16-bit storage, where an SM's own rate
@@ -192,6 +195,12 @@ struct Launch {
     // measured on GB300 (stream-collide, event-timed, FP32, nx x 64 x 64, tiles against
     // order) 33: 12.3 / 10.3 us, 110: 20.2 / 19.5, 120: 19.4 / 20.8, 240: 42.0 / 43.8; BF16
     // 165: 26.5 / 25.5.  The line lies at 7/8 of the lanes in use.
+    // Tiles sweep z within chunks of rows of kCellChunk cells a plane: over whole planes of
+    // 2^16 cells and more the z neighbours' stress and the populations streamed in z leave L2
+    // before the next plane comes (stream-collide, ps per cell, whole planes / chunks: FP32
+    // 256^2 36.0 / 34.5, 300^2 43.2 / 36.2, 384^2 38.1 / 34.3; BF16 256^2 31.2 / 28.1, 300^2
+    // 38.0 / 29.7, 384^2 30.3 / 28.1; half or a third of the chunk 1 to 3 % more).
+    static constexpr unsigned kCellChunk = sizeof(S) == 4 ? 3u << 14 : 3u << 13;
     template <class K, class... A>
     static cudaError_t cell_launch(const DevState &d, K tiled, K linear, cudaStream_t s, A... more) {
         const KArgs<S> a = args(d);
@@ -204,9 +213,17 @@ struct Launch {
             const unsigned t = std::max(32u, (a.lin / sms + 31u) / 32u * 32u);
             return launch_step(d.pdl, linear, dim3((a.lin + t - 1u) / t), dim3(t), 0, s, a, more...);
         }
-        const dim3 b = block2(d), g = grid2(d);
-        if (8LL * d.g.nx * d.g.ny >= 7LL * g.x * b.x * g.y * b.y)
+        const dim3 b = block2(d);
+        dim3 g = grid2(d);
+        if (8LL * d.g.nx * d.g.ny >= 7LL * g.x * b.x * g.y * b.y) {
+            const unsigned rows = std::max(1u, kCellChunk / ((unsigned)d.g.nx * b.y));
+            const unsigned chunks = (g.y + rows - 1u) / rows;
+            if (chunks > 1u && chunks * g.z <= 65535u) {
+                g.y = (g.y + chunks - 1u) / chunks;
+                g.z *= chunks;
+            }
             return launch_step(d.pdl, tiled, g, b, 0, s, a, more...);
+        }
         return launch_step(d.pdl, linear, dim3((a.lin + 127u) / 128u), dim3(128), 0, s, a, more...);
     }
     static cudaError_t lb(const DevState &d, int parity, cudaStream_t s) {
