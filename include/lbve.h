@@ -263,7 +263,7 @@ int lbve_is_unstable(const lbve_ctx *ctx);
  * row and the stress rows its polymer force reads (Eq. (force): the rows y -+ 1 and
  * z -+ 1) into shared memory with bulk asynchronous copies completing on mbarriers.  It
  * is taken with schedule PIPELINED (AUTO: from 2^22 cells, FP32 and 16-bit storage, for
- * row lengths of which an SM's shared memory holds 15 / 16 warps' worth) when
+ * row lengths of which an SM's shared memory holds 14 / 16 warps' worth) when
  * nx is a multiple of 32 in [64, 512], the PDF, stress and mask arrays are 16-byte
  * aligned (always with the library's own allocations), the layout fits one block's
  * shared memory (FP64: nx up to 384) and the stress law is not FENE-P.  LBVE_LB_CELLS:
