@@ -61,8 +61,8 @@ lbve_status lbve2d_init_fields(lbve2d_ctx *ctx, const double *rho, const double 
 
 /* Advance nsteps steps: polymer force and moments, finite-volume stress update, TRT
  * collision with forcing, push streaming with bounce-back.  Asynchronous.  Several steps on
- * a grid whose tiles are all resident run as one cooperative launch with a bounded grid
- * barrier per step; a wait that gave up makes later calls return LBVE_ETIMEOUT. */
+ * a grid whose tiles are all resident run as cooperative launches of up to 4096 steps with a
+ * bounded grid barrier per step; a wait that gave up makes later calls return LBVE_ETIMEOUT. */
 lbve_status lbve2d_step(lbve2d_ctx *ctx, int nsteps);
 
 /* rho (n), the physical velocity (j + F/2)/rho (2n), tau (3n); 0 in solid cells (each may

@@ -511,7 +511,8 @@ dim3 tiles2d(const lbve2d_ctx *c) {
     return dim3((unsigned)((c->p.nx + T2X - 1) / T2X), (unsigned)((c->p.ny + T2Y - 1) / T2Y));
 }
 
-// nsteps steps: one launch when every tile is resident, else two kernels per step.  The
+// nsteps steps: when every tile is resident, launches of up to GB_LAUNCH_STEPS steps, else
+// two kernels per step.  The
 // line is the device's (912 FP32 tiles on GB300, about 340^2 cells): beyond it the moments
 // computed twice and the blocks' waves cost more than the second launch (FP32 per step, this
 // kernel once per step against the two: 500^2 24.7 / 20.6 us, 1000^2 92 / 57).
@@ -523,17 +524,20 @@ cudaError_t step_impl(lbve2d_ctx *c, int nsteps) {
     if (nsteps > 1 && fits && !lbve::capturing(c->stream)) {
         cudaError_t e = multi_setup(c);
         if (e != cudaSuccess) return e;
-        Args2<R> a = args2<R>(c);
-        e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
-        if (e != cudaSuccess) return e;
-        void *args[] = {&a, &nsteps, &c->bar, &c->stuck_dev};
-        e = cudaLaunchCooperativeKernel((const void *)k2_steps<R, SH>, g, dim3(T2THREADS), args, 0, c->stream);
-        if (e != cudaSuccess) return e;
-        c->cur ^= nsteps & 1;
-        c->t += nsteps;
-        return cudaSuccess;
+        while (nsteps > 1) {
+            int m = lbve::launch_steps(nsteps, (long long)g.x * g.y);
+            Args2<R> a = args2<R>(c);
+            e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
+            if (e != cudaSuccess) return e;
+            void *args[] = {&a, &m, &c->bar, &c->stuck_dev};
+            e = cudaLaunchCooperativeKernel((const void *)k2_steps<R, SH>, g, dim3(T2THREADS), args, 0, c->stream);
+            if (e != cudaSuccess) return e;
+            c->cur ^= m & 1;
+            c->t += m;
+            nsteps -= m;
+        }
     }
-    for (int k = 0; k < nsteps; ++k) {
+    for (; nsteps > 0; --nsteps) {
         Args2<R> a = args2<R>(c);
         if (fits) {
             k2_steps<R, SH><<<g, T2THREADS, 0, c->stream>>>(a, 1, nullptr, nullptr);

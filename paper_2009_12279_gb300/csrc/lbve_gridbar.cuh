@@ -6,12 +6,24 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 namespace lbve {
 
 constexpr unsigned long long GB_WAIT_NS = 1000000000ull;  // 1 s
 
+// Steps that the next launch of a call takes when `steps` are left on a grid of `blocks`
+// blocks.  The barrier's word counts steps x blocks in 32 bits and must not wrap (a call of
+// 12.6 M steps on 343 blocks would), and a launch should end within tens of milliseconds;
+// 4096 steps of a few microseconds make the launch itself a few parts in ten thousand.
+constexpr int GB_LAUNCH_STEPS = 4096;
+inline int launch_steps(int steps, long long blocks) {
+    const long long most = std::min<long long>(GB_LAUNCH_STEPS, (1LL << 30) / std::max(1LL, blocks));
+    return (int)std::min<long long>(steps, std::max(1LL, most));
+}
+
 // Barrier number k (0, 1, ...) of the launch on a word that was 0 at its start: the blocks
-// count up to (k + 1) blocks.  False (in every thread of the block) when the wait gave up,
+// count up to (k + 1) blocks, at most 2^30 (launch_steps).  False (in every thread of the block) when the wait gave up,
 // after writing 2 to *status; the caller returns then.  The block barriers around the
 // release add and the acquire load make every thread's earlier writes visible to every
 // thread's later reads (PTX causality order); fences of their own would only add to it.
