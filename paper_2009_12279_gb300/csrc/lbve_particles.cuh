@@ -620,6 +620,37 @@ __device__ __forceinline__ void fill_drain(const PartEntry<S> &E, const KArgs<S>
     __syncthreads();
 }
 
+// The particles in `changed` and those that overlap or nearly touch one of them.  A cell that
+// a particle leaves inside another (spheres may overlap) has neighbours deep in that other
+// one, whose surface velocities are not kept up to date; it lies within R + 1 of the centre
+// it was left by, so the pairs closer than R_p + R_q + 1 + sqrt(2) matter.  FP32 with a cell
+// to spare; a lane per changed particle.
+__device__ __forceinline__ unsigned long long with_touching(const Geo &g, const PartDev *parts, int nparts,
+                                                            unsigned long long changed) {
+    unsigned long long out = changed;
+    if (!changed) return out;
+    const int nn[3] = {g.nx, g.ny, g.nz};
+#pragma unroll 1
+    for (int p = 0; p < nparts; ++p) {
+        if ((changed >> p) & 1ull) continue;
+        bool near = false;
+#pragma unroll 1
+        for (int q = (int)threadIdx.x & 31; q < nparts; q += 32) {
+            if (!((changed >> q) & 1ull)) continue;
+            float d2 = 0.0f;
+            for (int k = 0; k < 3; ++k) {
+                float d = (float)parts[p].X[k] - (float)parts[q].X[k];
+                if (g.per[k]) d -= (float)nn[k] * rintf(d / (float)nn[k]);
+                d2 += d * d;
+            }
+            const float reach = (float)parts[p].R + (float)parts[q].R + 3.5f;
+            near |= d2 <= reach * reach;
+        }
+        if (__any_sync(0xffffffffu, near)) out |= 1ull << p;
+    }
+    return out;
+}
+
 // Particle phase of one step for one solve per cluster: sums of the momentum-exchange
 // partials (reduced modes), symplectic Euler, fill/drain of the cells the spheres now cover
 // or have left (the particles one after another), links of the particles whose cells
@@ -698,8 +729,8 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
                 const bool inside = inside_sphere(a.g, P, sf, x, y, z, d2);
                 kd = old == FLAG_FLUID ? (inside ? 2 : 1) : (inside ? 0 : 3);
                 // the surface velocity of a cell the sphere keeps (again below when
-                // conversions change the sphere's velocity).  A cell deeper than sqrt(2)
-                // below the surface has no fluid neighbour to read it.
+                // conversions change the sphere's velocity or free a cell inside it).  A cell
+                // deeper than sqrt(2) below the surface has no fluid neighbour to read it.
                 if (kd == 0 && d2 >= sf.deep2) set_solid_velocity<S>(a, x, y, z, r, a.u_out, a.u_out);
             }
             E.kind[q] = (uint8_t)kd;
@@ -737,9 +768,10 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(PT)
         }
         cl.sync();
     }
-    // surface velocities of the spheres whose velocity the conversions changed
+    // surface velocities of the spheres whose velocity or neighbourhood the conversions changed
+    const unsigned long long redo = with_touching(a.g, E.parts, E.nparts, changed);
     for (int p = E.nparts - 1; p >= 0; --p) {
-        if (!((changed >> p) & 1ull)) continue;
+        if (!((redo >> p) & 1ull)) continue;
         if (p + 1 < E.nparts) {  // the box of the last particle is still there
             __syncthreads();
             if (warp == 0) prepare_box(a.g, E.parts[p], 3, w, nullptr);
