@@ -279,9 +279,8 @@ namespace {
 // Sum the momentum-exchange contributions of each body segment in link order (FP64
 // parity mode, launched with one thread per body: the sequential order of a plain loop;
 // with more threads a fixed-shape block reduction).
-__global__ void k_body_reduce(const double *__restrict__ contrib, const int *__restrict__ seg_begin,
-                              const int *__restrict__ seg_count, const int *__restrict__ seg_flag, int nbody,
-                              double *__restrict__ body_F, PartDev *__restrict__ parts) {
+__global__ void k_body_reduce(const double *contrib, const int *__restrict__ seg_begin, const int *seg_count,
+                              const int *__restrict__ seg_flag, int nbody, double *body_F, PartDev *parts) {
     step_wait();
     step_next();
     const int b = blockIdx.x;
@@ -316,10 +315,9 @@ __global__ void k_body_reduce(const double *__restrict__ contrib, const int *__r
 // Per-body sums of the reduced modes' momentum-exchange partials (gx per body, first
 // ceil(count / 128) used): warp w sums component w over partials lane, lane + 32, ...,
 // then a fixed shuffle tree.  Deterministic.
-__global__ void __launch_bounds__(192) k_body_partials(const double *__restrict__ part, int gx,
-                                                       const int *__restrict__ seg_count,
-                                                       const int *__restrict__ seg_flag, int nbody,
-                                                       double *__restrict__ body_F, PartDev *__restrict__ parts) {
+__global__ void __launch_bounds__(192) k_body_partials(const double *part, int gx, const int *seg_count,
+                                                       const int *__restrict__ seg_flag, int nbody, double *body_F,
+                                                       PartDev *parts) {
     step_wait();
     step_next();
     const int b = blockIdx.x;

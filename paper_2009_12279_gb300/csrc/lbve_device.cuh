@@ -354,7 +354,7 @@ __device__ __forceinline__ void polymer_force_core_fene(const R (&tr)[6], uint32
 // Same with the stress read from global memory (the FENE-P form when ph.fene).
 template <class R>
 __device__ __forceinline__ void polymer_force(const Geo &g, const Phys<R> &ph, const Cell &cl, unsigned r,
-                                              uint32_t mask, const R *__restrict__ tau, R Fp[3]) {
+                                              uint32_t mask, const R *tau, R Fp[3]) {
     const size_t np = (size_t)g.np;
     R tr[6];
 #pragma unroll

@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(256) k_residual(Geo g, const uint32_t *__restr
 // ---------------------------------------------------------------------------------
 // Momentum-exchange contribution of one link (code = r << 5 | i) into contrib[8].
 template <class S, int PAR>
-__device__ __forceinline__ void me_link(const KArgs<S> &a, long long code, double *__restrict__ o) {
+__device__ __forceinline__ void me_link(const KArgs<S> &a, long long code, double *o) {
     using R = typename Store<S>::R;
     constexpr bool SH = Store<S>::shifted;
     const int i = (int)(code & 31);
@@ -1231,10 +1231,9 @@ __device__ __forceinline__ void me_link(const KArgs<S> &a, long long code, doubl
 // Momentum exchange over link segments (one segment per tracked body, blockIdx.y):
 // link l of segment b is links[seg_begin[b] + l] for l < seg_count[b].
 template <class S, int PAR>
-__global__ void __launch_bounds__(128) k_momentum_exchange(KArgs<S> a, const long long *__restrict__ links,
-                                                           const int *__restrict__ seg_begin,
-                                                           const int *__restrict__ seg_count,
-                                                           double *__restrict__ contrib) {
+__global__ void __launch_bounds__(128) k_momentum_exchange(KArgs<S> a, const long long *links,
+                                                           const int *__restrict__ seg_begin, const int *seg_count,
+                                                           double *contrib) {
     step_wait();
     const int b = blockIdx.y;
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1247,10 +1246,9 @@ __global__ void __launch_bounds__(128) k_momentum_exchange(KArgs<S> a, const lon
 // of 6 doubles (stride 8) per (body, block) at part[(b * gridDim.x + block) * 8].  The
 // final per-body sum then reads ceil(count / 128) partials instead of every link.
 template <class S, int PAR>
-__global__ void __launch_bounds__(128) k_momentum_exchange_part(KArgs<S> a, const long long *__restrict__ links,
+__global__ void __launch_bounds__(128) k_momentum_exchange_part(KArgs<S> a, const long long *links,
                                                                 const int *__restrict__ seg_begin,
-                                                                const int *__restrict__ seg_count,
-                                                                double *__restrict__ part) {
+                                                                const int *seg_count, double *part) {
     step_wait();
     step_next();
     const int b = blockIdx.y;

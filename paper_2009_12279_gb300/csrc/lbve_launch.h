@@ -115,7 +115,10 @@ struct DevState {
 #ifdef __CUDACC__
 // A step kernel may be launched before its predecessor in the stream has finished: it waits
 // here, before it reads or writes anything, until that one is complete and its writes are
-// visible.  Every thread of every step kernel passes here first.
+// visible.  Every thread of every step kernel passes here first.  What its predecessors write
+// changes during its own lifetime, so no step kernel takes an array that a step kernel writes
+// as `const ... *__restrict__`: that would promise the compiler that nobody does, and allow it
+// a non-coherent load or one above this wait.
 __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // ... and lets its own successor be launched once all its blocks have come here.  After
 // a block's loads, not at its start: blocks that wait from early on take the slots of, and
