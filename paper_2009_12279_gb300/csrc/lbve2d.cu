@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(T2THREADS) k2_steps(Args2<R> a, int nsteps, un
         } else if (own && used) {
             for (int c = 0; c < 3; ++c) a.tau_out[c * a.n + r] = R(0);
         }
-        if (s + 1 == nsteps || !lbve::grid_barrier(bar, (unsigned)s, status)) return;
+        if (s + 1 == nsteps || !lbve::grid_barrier(bar, (unsigned)s, gridDim.x * gridDim.y, status)) return;
         const R *ft = a.f_in, *tt = a.tau;
         a.f_in = a.f_out;
         a.f_out = const_cast<R *>(ft);

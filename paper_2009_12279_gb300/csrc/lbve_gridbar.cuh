@@ -10,7 +10,12 @@
 
 namespace lbve {
 
-constexpr unsigned long long GB_WAIT_NS = 1000000000ull;  // 1 s
+// Limits of a barrier's wait.  At the launch's first barrier some blocks may not have started
+// yet, held up by another stream's kernel on their SMs; from then on all of them are resident
+// and a step takes microseconds.
+constexpr unsigned long long GB_FIRST_NS = 20000000000ull;  // 20 s
+constexpr unsigned long long GB_WAIT_NS = 1000000000ull;    // 1 s
+constexpr unsigned GB_LEFT = 1u << 31;  // set in the word by a block that gave up
 
 // Steps that the next launch of a call takes when `steps` are left on a grid of `blocks`
 // blocks.  The barrier's word counts steps x blocks in 32 bits and must not wrap (a call of
@@ -22,29 +27,38 @@ inline int launch_steps(int steps, long long blocks) {
     return (int)std::min<long long>(steps, std::max(1LL, most));
 }
 
-// Barrier number k (0, 1, ...) of the launch on a word that was 0 at its start: the blocks
-// count up to (k + 1) blocks, at most 2^30 (launch_steps).  False (in every thread of the block) when the wait gave up,
-// after writing 2 to *status; the caller returns then.  The block barriers around the
-// release add and the acquire load make every thread's earlier writes visible to every
-// thread's later reads (PTX causality order); fences of their own would only add to it.
-__device__ __forceinline__ bool grid_barrier(unsigned *word, unsigned k, unsigned *status) {
+// Barrier number k (0, 1, ...) of `blocks` blocks on a word that was 0 at the launch's start:
+// they count up to (k + 1) blocks, at most 2^30 (launch_steps).  False (in every thread of
+// the block) when the wait gave up, after writing 2 to *status and marking the word, or when
+// another block did: the caller returns then, and so do the others, at this barrier or the
+// next.  The block barriers around the release add and the acquire load make every thread's
+// earlier writes visible to every thread's later reads (PTX causality order); fences of their
+// own would only add to it.
+__device__ __forceinline__ bool grid_barrier(unsigned *word, unsigned k, unsigned blocks, unsigned *status,
+                                             unsigned long long first_ns = GB_FIRST_NS,
+                                             unsigned long long wait_ns = GB_WAIT_NS) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0 && threadIdx.y == 0) {
-        const unsigned blocks = gridDim.x * gridDim.y * gridDim.z, target = (k + 1u) * blocks;
+        const unsigned target = (k + 1u) * blocks;
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
+        const unsigned long long limit = k == 0 ? first_ns : wait_ns;
         unsigned long long t0 = 0;
         ok = 1;
         for (unsigned n = 0;; ++n) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
-            if (v >= target) break;
+            if (v >= target) {
+                ok = v < GB_LEFT;
+                break;
+            }
             if ((n & 255u) == 255u) {
                 unsigned long long t;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
                 if (t0 == 0)
                     t0 = t;
-                else if (t - t0 > GB_WAIT_NS) {
+                else if (t - t0 > limit) {
+                    atomicOr(word, GB_LEFT);
                     if (status) *(volatile unsigned *)status = 2u;
                     ok = 0;
                     break;
