@@ -413,8 +413,9 @@ struct lbve2d_ctx {
     size_t rb = 8;
     void *f[2] = {nullptr, nullptr}, *tau[2] = {nullptr, nullptr}, *u = nullptr, *ub = nullptr, *force = nullptr;
     uint8_t *flag = nullptr;
-    double *stage = nullptr;  // FP64 staging, 10 n doubles
-    // set up by the first call that takes several steps in one launch:
+    double *stage = nullptr;  // FP64 staging, 15 n doubles
+    void *arena = nullptr;    // the one device allocation that holds all of these but force
+    // multi-step launches; here from creation on, so that lbve2d_step allocates nothing
     unsigned *bar = nullptr;    // device word of the grid barrier
     unsigned *stuck = nullptr;  // mapped host word: 2 once a barrier's bounded wait gave up
     unsigned *stuck_dev = nullptr;
@@ -490,23 +491,6 @@ const char *const kStuck = "the blocks of a multi-step launch gave up waiting fo
 dim3 block2d() { return dim3(64, 2); }
 dim3 grid2d(const lbve2d_ctx *c) { return dim3((unsigned)((c->p.nx + 63) / 64), (unsigned)((c->p.ny + 1) / 2)); }
 
-cudaError_t multi_setup(lbve2d_ctx *c) {
-    if (c->stuck) return cudaSuccess;
-    cudaError_t e = c->bar ? cudaSuccess : cudaMalloc((void **)&c->bar, sizeof(unsigned));
-    if (e != cudaSuccess) return e;
-    unsigned *w = nullptr;
-    e = cudaHostAlloc((void **)&w, sizeof(unsigned), cudaHostAllocMapped);
-    if (e != cudaSuccess) return e;
-    *w = 0u;
-    e = cudaHostGetDevicePointer((void **)&c->stuck_dev, w, 0);
-    if (e != cudaSuccess) {
-        cudaFreeHost(w);
-        return e;
-    }
-    c->stuck = w;
-    return cudaSuccess;
-}
-
 dim3 tiles2d(const lbve2d_ctx *c) {
     return dim3((unsigned)((c->p.nx + T2X - 1) / T2X), (unsigned)((c->p.ny + T2Y - 1) / T2Y));
 }
@@ -522,12 +506,10 @@ cudaError_t step_impl(lbve2d_ctx *c, int nsteps) {
     if (c->resident < 0) c->resident = lbve::resident_blocks(k2_steps<R, SH>, T2THREADS, 0);
     const bool fits = (long long)g.x * g.y <= c->resident;
     if (nsteps > 1 && fits && !lbve::capturing(c->stream)) {
-        cudaError_t e = multi_setup(c);
-        if (e != cudaSuccess) return e;
         while (nsteps > 1) {
             int m = lbve::launch_steps(nsteps, (long long)g.x * g.y);
             Args2<R> a = args2<R>(c);
-            e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
+            cudaError_t e = cudaMemsetAsync(c->bar, 0, sizeof(unsigned), c->stream);
             if (e != cudaSuccess) return e;
             void *args[] = {&a, &m, &c->bar, &c->stuck_dev};
             e = cudaLaunchCooperativeKernel((const void *)k2_steps<R, SH>, g, dim3(T2THREADS), args, 0, c->stream);
@@ -615,13 +597,34 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
     ph.flux_on = (terms & LBVE_FV_FLUX) != 0;
     ph.src_on = (terms & LBVE_FV_SOURCE) != 0;
     const size_t n = (size_t)c->n;
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMalloc(&c->f[k], Q2 * n * c->rb);
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMalloc(&c->tau[k], 3 * n * c->rb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->u, 2 * n * c->rb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->ub, 2 * n * c->rb);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->flag, n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->stage, 15 * n * sizeof(double));
+    size_t bytes = 0;
+    auto take = [&](size_t b) {
+        const size_t at = bytes;
+        bytes += (b + 255) / 256 * 256;
+        return at;
+    };
+    const size_t at_f[2] = {take(Q2 * n * c->rb), take(Q2 * n * c->rb)};
+    const size_t at_tau[2] = {take(3 * n * c->rb), take(3 * n * c->rb)};
+    const size_t at_u = take(2 * n * c->rb), at_ub = take(2 * n * c->rb), at_flag = take(n);
+    const size_t at_stage = take(15 * n * sizeof(double)), at_bar = take(sizeof(unsigned));
+    cudaError_t e = cudaMalloc(&c->arena, bytes);
+    if (e == cudaSuccess) {
+        char *p0 = (char *)c->arena;
+        for (int k = 0; k < 2; ++k) {
+            c->f[k] = p0 + at_f[k];
+            c->tau[k] = p0 + at_tau[k];
+        }
+        c->u = p0 + at_u;
+        c->ub = p0 + at_ub;
+        c->flag = (uint8_t *)(p0 + at_flag);
+        c->stage = (double *)(p0 + at_stage);
+        c->bar = (unsigned *)(p0 + at_bar);
+        e = cudaHostAlloc((void **)&c->stuck, sizeof(unsigned), cudaHostAllocMapped);
+    }
+    if (e == cudaSuccess) {
+        *c->stuck = 0u;
+        e = cudaHostGetDevicePointer((void **)&c->stuck_dev, c->stuck, 0);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->flag, 0, n, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->ub, 0, 2 * n * c->rb, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->u, 0, 2 * n * c->rb, c->stream);
@@ -646,8 +649,7 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
 lbve_status lbve2d_destroy(lbve2d_ctx *c) {
     if (!c) return LBVE_EINVAL;
     cudaStreamSynchronize(c->stream);
-    for (void *p : {c->f[0], c->f[1], c->tau[0], c->tau[1], c->u, c->ub, c->force, (void *)c->flag, (void *)c->stage,
-                    (void *)c->bar})
+    for (void *p : {c->arena, c->force})
         if (p) cudaFree(p);
     if (c->stuck) cudaFreeHost(c->stuck);
     delete c;
