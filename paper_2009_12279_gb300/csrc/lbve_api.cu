@@ -1485,10 +1485,11 @@ struct lbve_pool {
     // residual staging
     double *res_dev = nullptr;
     size_t res_cap = 0;
-    // CUDA graphs, one per call parity
+    // CUDA graphs per call parity (see lbve_pool_step): [0] a block of steps in the middle of a
+    // call, [1] the last steps of one, with the number of steps each was captured for
     bool use_graphs = true;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    int graph_steps[2] = {0, 0};
+    cudaGraphExec_t graph[2][2] = {};
+    int graph_steps[2][2] = {};
     // side streams: the members' small per-step kernels (momentum exchange, body sums,
     // particle update, fill/drain, links) touch only their own buffers, so the chains of
     // different members run side by side, forked from and joined back to the pool stream
@@ -1514,10 +1515,10 @@ lbve_status pfail(lbve_pool *P, lbve_status s, const std::string &m) {
     } while (0)
 
 void drop_graphs(lbve_pool *P) {
-    for (int k = 0; k < 2; ++k) {
-        if (P->graph[k]) cudaGraphExecDestroy(P->graph[k]);
-        P->graph[k] = nullptr;
-        P->graph_steps[k] = 0;
+    for (int k = 0; k < 4; ++k) {
+        if (P->graph[k >> 1][k & 1]) cudaGraphExecDestroy(P->graph[k >> 1][k & 1]);
+        P->graph[k >> 1][k & 1] = nullptr;
+        P->graph_steps[k >> 1][k & 1] = 0;
     }
 }
 
@@ -1691,16 +1692,17 @@ lbve_status member_bodies(lbve_pool *P, lbve_ctx *c, const DevState &d, int pari
     return LBVE_OK;
 }
 
-// A member's whole call on a stream of its own (members do not depend on one another).
-lbve_status enqueue_own(lbve_pool *P, lbve_ctx *c, int nsteps, cudaStream_t st) {
+// A member's steps on a stream of its own (members do not depend on one another); last: they
+// end the call.
+lbve_status enqueue_own(lbve_pool *P, lbve_ctx *c, int nsteps, bool last, cudaStream_t st) {
     DevState d = c->d;
     d.in_pool = 1;
     d.dstep = P->dstep + 1;
     for (int k = 0; k < nsteps; ++k) {
         const int parity = (int)((c->t + k) & 1);
-        // at the call, *dstep is the number of steps since the build (now and in replays)
+        // *dstep is the number of steps since the build when these begin (now and in replays)
         d.step = (unsigned)(c->t - P->steps_since_build + k);
-        if (c->nbody > 0 && (c->nparts > 0 || k + 1 == nsteps)) {
+        if (c->nbody > 0 && (c->nparts > 0 || (last && k + 1 == nsteps))) {
             lbve_status s = member_bodies(P, c, d, parity, st);
             if (s != LBVE_OK) return s;
         }
@@ -1712,15 +1714,15 @@ lbve_status enqueue_own(lbve_pool *P, lbve_ctx *c, int nsteps, cudaStream_t st) 
     return LBVE_OK;
 }
 
-// Enqueue nsteps steps of every member on the pool stream (graph-capturable): the large
-// members' calls on the lower half of the side streams, the others together by the batched
+// Enqueue nsteps steps of every member on the pool stream (graph-capturable), the last of a
+// call or not: the large members' steps on the lower half of the side streams, the others together by the batched
 // kernels, their momentum exchange on the upper half.
-lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
+lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps, bool last) {
     const int n_own = std::min<int>(P->batch.empty() ? lbve_pool::kSide : lbve_pool::kSide / 2, (int)P->own.size());
     if (n_own > 0) {
         lbve_status s = side_fork(P, 0, n_own);
         for (size_t i = 0; i < P->own.size() && s == LBVE_OK; ++i)
-            s = enqueue_own(P, P->own[i], nsteps, P->side[i % (size_t)n_own]);
+            s = enqueue_own(P, P->own[i], nsteps, last, P->side[i % (size_t)n_own]);
         if (s != LBVE_OK) return s;
     }
     std::vector<lbve_ctx *> with_bodies;
@@ -1729,7 +1731,7 @@ lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
         // members with wall classes only: the forces of the call's last step (see lbve_step)
         with_bodies.clear();
         for (lbve_ctx *c : P->batch)
-            if (c->nbody > 0 && (c->nparts > 0 || k + 1 == nsteps)) with_bodies.push_back(c);
+            if (c->nbody > 0 && (c->nparts > 0 || (last && k + 1 == nsteps))) with_bodies.push_back(c);
         lbve_status s = fan_out(P, with_bodies, lbve_pool::kSide / 2, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
             DevState d = c->d;  // the member's state at the start of this call
             if (k & 1) d.cur ^= 1;
@@ -1759,6 +1761,34 @@ lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps) {
         k_step_count<<<1, 1, 0, P->stream>>>(P->dstep + 1, (unsigned)nsteps);
         PCK(cudaGetLastError(), "step counter");
     }
+    return LBVE_OK;
+}
+
+// Kernels that a step of the pool enqueues.
+long long step_nodes(const lbve_pool *P) {
+    long long n = P->own.empty() ? 0 : 2;
+    auto bodies = [](const lbve_ctx *c) { return c->nparts > 0 ? (phase_sums(c) ? 1 : 2) : 0; };
+    for (const lbve_ctx *c : P->own) n += 2 + bodies(c) + (c->nparts > 0 ? 1 : 0);
+    if (!P->batch.empty()) n += 4 + (long long)P->fv_groups.size();
+    for (const lbve_ctx *c : P->batch) n += bodies(c);
+    return n;
+}
+
+// Capture nsteps steps into P->graph[q][last] unless it holds them.
+lbve_status capture_steps(lbve_pool *P, int q, int nsteps, bool last) {
+    cudaGraphExec_t &exec = P->graph[q][last];
+    if (exec && P->graph_steps[q][last] == nsteps) return LBVE_OK;
+    if (exec) cudaGraphExecDestroy(exec);
+    exec = nullptr;
+    cudaGraph_t g;
+    PCK(cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
+    lbve_status s = enqueue_steps(P, q, nsteps, last);
+    cudaError_t e = cudaStreamEndCapture(P->stream, &g);
+    if (s != LBVE_OK) return s;
+    PCK(e, "end capture");
+    PCK(cudaGraphInstantiate(&exec, g, 0), "graph instantiate");
+    cudaGraphDestroy(g);
+    P->graph_steps[q][last] = nsteps;
     return LBVE_OK;
 }
 
@@ -1865,22 +1895,17 @@ lbve_status lbve_pool_step(lbve_pool *P, int nsteps) {
     }
     const int q = (int)(P->steps_since_build & 1);
     if (pool_graphs(P)) {
-        if (!P->graph[q] || P->graph_steps[q] != nsteps) {
-            if (P->graph[q]) cudaGraphExecDestroy(P->graph[q]);
-            P->graph[q] = nullptr;
-            cudaGraph_t g;
-            PCK(cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-            lbve_status s = enqueue_steps(P, q, nsteps);
-            cudaError_t e = cudaStreamEndCapture(P->stream, &g);
-            if (s != LBVE_OK) return s;
-            PCK(e, "end capture");
-            PCK(cudaGraphInstantiate(&P->graph[q], g, 0), "graph instantiate");
-            cudaGraphDestroy(g);
-            P->graph_steps[q] = nsteps;
-        }
-        PCK(cudaGraphLaunch(P->graph[q], P->stream), "graph launch");
+        // A call longer than a block of graph_block_steps() steps replays a graph of that many
+        // (an even number: parities and ping-pongs return to where they were) and ends with
+        // one of the remaining 1 to block steps, which includes the forces on wall classes.
+        const int block = graph_block_steps(step_nodes(P)), blocks = (nsteps - 1) / block;
+        lbve_status s = blocks > 0 ? capture_steps(P, q, block, false) : LBVE_OK;
+        if (s == LBVE_OK) s = capture_steps(P, q, nsteps - blocks * block, true);
+        if (s != LBVE_OK) return s;
+        for (int b = 0; b < blocks; ++b) PCK(cudaGraphLaunch(P->graph[q][0], P->stream), "graph launch");
+        PCK(cudaGraphLaunch(P->graph[q][1], P->stream), "graph launch");
     } else {
-        lbve_status s = enqueue_steps(P, q, nsteps);
+        lbve_status s = enqueue_steps(P, q, nsteps, true);
         if (s != LBVE_OK) return s;
     }
     for (lbve_ctx *c : P->members) {

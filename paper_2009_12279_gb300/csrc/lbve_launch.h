@@ -146,6 +146,18 @@ inline cudaError_t launch_step(int pdl, void (*kernel)(P...), dim3 grid, dim3 bl
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
+// Steps of a pool's replayed graph, an even number, for steps of `nodes` kernels each: about
+// GRAPH_NODES kernels to capture, instantiate and keep, however long a call is.  48 members of
+// the serving mix, BF16, ms of the first call after an admission and of a replay: 100 steps in
+// one graph 113 / 68.2, blocks of 1024 kernels 72 / 68.3, 2048 75 / 68.0, 4096 83 / 68.2, 8192
+// 114 / 68.0; 1000 steps 1198 / 687 (402 MB on the device), 690 / 684, 691 / 679 (55 MB), 704 /
+// 683, 736 / 684.
+constexpr long long GRAPH_NODES = 2048;
+inline int graph_block_steps(long long nodes) {
+    const long long steps = GRAPH_NODES / (nodes > 0 ? nodes : 1);
+    return (int)(steps < 2 ? 2 : steps / 2 * 2);
+}
+
 struct KernelTable {
     int prec;          // lbve_pdf_prec
     size_t pdf_bytes;  // bytes per stored PDF
