@@ -1374,18 +1374,27 @@ static int residual_blocks(const lbve_ctx *c) {
     return (int)(b > 1024 ? 1024 : (b < 1 ? 1 : b));
 }
 
-// Block partials of the residual into `partial` (nullptr: the context's own buffer) on a
-// stream that follows the context's.
-static lbve_status residual_enqueue(lbve_ctx *c, double *partial = nullptr, cudaStream_t st = nullptr) {
-    const int nb = residual_blocks(c);
-    if (!partial) st = c->stream;
-    if (!c->usnap) {
-        c->usnap = dev_alloc(c, (size_t)3 * c->d.g.np * c->kt->real_bytes);
-        c->res_partial = (double *)dev_alloc(c, sizeof(double) * 2 * 1024);
-        if (!c->usnap || !c->res_partial) return fail(c, LBVE_ENOMEM, "residual buffers");
-        CK(cudaMemsetAsync(c->usnap, 0, (size_t)3 * c->d.g.np * c->kt->real_bytes, st), "residual clear");
+// The residual's buffers, made by the first call: all of them or none.
+static lbve_status residual_buffers(lbve_ctx *c) {
+    if (c->usnap) return LBVE_OK;
+    const size_t bytes = (size_t)3 * c->d.g.np * c->kt->real_bytes;
+    void *snap = dev_alloc(c, bytes);
+    double *partial = (double *)dev_alloc(c, sizeof(double) * 2 * 1024);
+    const cudaError_t e = snap && partial ? cudaMemsetAsync(snap, 0, bytes, c->stream) : cudaSuccess;
+    if (!snap || !partial || e != cudaSuccess) {
+        dev_free(c, snap);
+        dev_free(c, partial);
+        CK(e, "residual clear");
+        return fail(c, LBVE_ENOMEM, "residual buffers");
     }
-    CK(c->kt->residual(c->d, c->usnap, partial ? partial : c->res_partial, nb, st), "residual kernel");
+    c->usnap = snap;
+    c->res_partial = partial;
+    return LBVE_OK;
+}
+
+// Block partials of the residual into `partial`, on a stream that follows the context's.
+static lbve_status residual_enqueue(lbve_ctx *c, double *partial, cudaStream_t st) {
+    CK(c->kt->residual(c->d, c->usnap, partial, residual_blocks(c), st), "residual kernel");
     return LBVE_OK;
 }
 
@@ -1402,7 +1411,8 @@ static void residual_finish(const lbve_ctx *c, const double *partial, double out
 
 lbve_status lbve_residual(lbve_ctx *c, double out[2]) {
     if (!c || !out) return c ? fail(c, LBVE_EINVAL, "out is NULL") : LBVE_EINVAL;
-    lbve_status s = residual_enqueue(c);
+    lbve_status s = residual_buffers(c);
+    if (s == LBVE_OK) s = residual_enqueue(c, c->res_partial, c->stream);
     if (s != LBVE_OK) return s;
     std::vector<double> h(2 * 1024);
     CK(cudaMemcpyAsync(h.data(), c->res_partial, sizeof(double) * 2 * residual_blocks(c), cudaMemcpyDeviceToHost,
@@ -1666,8 +1676,19 @@ lbve_status side_join(lbve_pool *P, int first, int count) {
     return LBVE_OK;
 }
 
+// The status of forked work, joined: the first error, if any.
+lbve_status joined(lbve_pool *P, lbve_status s, int first, int count) {
+    const std::string err = P->err;
+    const lbve_status j = side_join(P, first, count);
+    if (s == LBVE_OK) return j;
+    P->err = err;
+    return s;
+}
+
 // Run body(member, stream) for every listed member: on the pool stream when there is one
-// member, else spread over the side streams from `first` on between a fork and a join.
+// member, else spread over the side streams from `first` on between a fork and a join.  What
+// was forked is joined whatever failed in between (here and in enqueue_steps): work that the
+// side streams hold stays ordered before the pool stream's, and a capture can be ended.
 template <class Body>
 lbve_status fan_out(lbve_pool *P, const std::vector<lbve_ctx *> &list, int first, Body &&body) {
     const int ns = std::min<int>(lbve_pool::kSide - first, (int)list.size());
@@ -1680,8 +1701,7 @@ lbve_status fan_out(lbve_pool *P, const std::vector<lbve_ctx *> &list, int first
     }
     lbve_status s = side_fork(P, first, ns);
     for (size_t i = 0; i < list.size() && s == LBVE_OK; ++i) s = body(list[i], P->side[first + (int)(i % ns)]);
-    if (s != LBVE_OK) return s;
-    return side_join(P, first, ns);
+    return joined(P, s, first, ns);
 }
 
 lbve_status member_bodies(lbve_pool *P, lbve_ctx *c, const DevState &d, int parity, cudaStream_t st) {
@@ -1714,53 +1734,53 @@ lbve_status enqueue_own(lbve_pool *P, lbve_ctx *c, int nsteps, bool last, cudaSt
     return LBVE_OK;
 }
 
+// Step k of nsteps of the members that share the batched kernels; their momentum exchange on
+// the upper half of the side streams.
+lbve_status enqueue_batch(lbve_pool *P, int q, int k, bool forces) {
+    const int kk = q + k;  // steps since the entries were built (they encode that state)
+    // members with wall classes only: the forces of the call's last step (see lbve_step)
+    std::vector<lbve_ctx *> with_bodies;
+    for (lbve_ctx *c : P->batch)
+        if (c->nbody > 0 && (c->nparts > 0 || forces)) with_bodies.push_back(c);
+    lbve_status s = fan_out(P, with_bodies, lbve_pool::kSide / 2, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
+        DevState d = c->d;  // the member's state at the start of these steps
+        if (k & 1) d.cur ^= 1;
+        return member_bodies(P, c, d, (int)((c->t + k) & 1), st);
+    });
+    if (s != LBVE_OK) return s;
+    for (int par = 0; par < 2; ++par) {  // the group of build parity par is at parity (par + kk) & 1
+        const lbve_pool::LbClass &cl = P->lb_class[par];
+        if (cl.n == 0) continue;
+        PCK(P->kt->lb_batched((const unsigned char *)P->entries[1] + (size_t)cl.start * P->kt->batch_entry_bytes, cl.n,
+                              cl.total, kk, P->grid_lb, P->dstep, (par + kk) & 1, P->stream),
+            "batched lb");
+    }
+    k_step_count<<<1, 1, 0, P->stream>>>(P->dstep, 1u);
+    PCK(cudaGetLastError(), "step counter");
+    for (const lbve_pool::FvGroup &grp : P->fv_groups)
+        PCK(P->kt->fv_batched((const unsigned char *)P->entries[0] + (size_t)grp.start * P->kt->batch_entry_bytes, grp.n,
+                              grp.total, kk, grp.grid, grp.tx, grp.var, P->stream),
+            "batched fv");
+    // particle update, fill/drain and links of every batched member with particles: one
+    // cluster per member in one launch
+    PCK(P->kt->particle_phase_batched(P->pentries, P->n_pentries, kk, P->stream), "pool particle phase");
+    return LBVE_OK;
+}
+
 // Enqueue nsteps steps of every member on the pool stream (graph-capturable), the last of a
-// call or not: the large members' steps on the lower half of the side streams, the others together by the batched
-// kernels, their momentum exchange on the upper half.
+// call or not: the members with kernels of their own on the side streams (their lower half
+// when there are others), the others together by the batched kernels.
 lbve_status enqueue_steps(lbve_pool *P, int q, int nsteps, bool last) {
     const int n_own = std::min<int>(P->batch.empty() ? lbve_pool::kSide : lbve_pool::kSide / 2, (int)P->own.size());
-    if (n_own > 0) {
-        lbve_status s = side_fork(P, 0, n_own);
-        for (size_t i = 0; i < P->own.size() && s == LBVE_OK; ++i)
-            s = enqueue_own(P, P->own[i], nsteps, last, P->side[i % (size_t)n_own]);
-        if (s != LBVE_OK) return s;
-    }
-    std::vector<lbve_ctx *> with_bodies;
-    for (int k = 0; k < nsteps && !P->batch.empty(); ++k) {
-        const int kk = q + k;  // steps since the entries were built (they encode that state)
-        // members with wall classes only: the forces of the call's last step (see lbve_step)
-        with_bodies.clear();
-        for (lbve_ctx *c : P->batch)
-            if (c->nbody > 0 && (c->nparts > 0 || (last && k + 1 == nsteps))) with_bodies.push_back(c);
-        lbve_status s = fan_out(P, with_bodies, lbve_pool::kSide / 2, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
-            DevState d = c->d;  // the member's state at the start of this call
-            if (k & 1) d.cur ^= 1;
-            return member_bodies(P, c, d, (int)((c->t + k) & 1), st);
-        });
-        if (s != LBVE_OK) return s;
-        for (int par = 0; par < 2; ++par) {  // the group of build parity par is at parity (par + kk) & 1
-            const lbve_pool::LbClass &cl = P->lb_class[par];
-            if (cl.n == 0) continue;
-            PCK(P->kt->lb_batched((const unsigned char *)P->entries[1] + (size_t)cl.start * P->kt->batch_entry_bytes,
-                                  cl.n, cl.total, kk, P->grid_lb, P->dstep, (par + kk) & 1, P->stream),
-                "batched lb");
-        }
-        k_step_count<<<1, 1, 0, P->stream>>>(P->dstep, 1u);
-        PCK(cudaGetLastError(), "step counter");
-        for (const lbve_pool::FvGroup &grp : P->fv_groups)
-            PCK(P->kt->fv_batched((const unsigned char *)P->entries[0] + (size_t)grp.start * P->kt->batch_entry_bytes,
-                                  grp.n, grp.total, kk, grp.grid, grp.tx, grp.var, P->stream),
-                "batched fv");
-        // particle update, fill/drain and links of every batched member with particles: one
-        // cluster per member in one launch
-        PCK(P->kt->particle_phase_batched(P->pentries, P->n_pentries, kk, P->stream), "pool particle phase");
-    }
-    if (n_own > 0) {
-        lbve_status s = side_join(P, 0, n_own);
-        if (s != LBVE_OK) return s;
-        k_step_count<<<1, 1, 0, P->stream>>>(P->dstep + 1, (unsigned)nsteps);
-        PCK(cudaGetLastError(), "step counter");
-    }
+    lbve_status s = n_own > 0 ? side_fork(P, 0, n_own) : LBVE_OK;
+    for (size_t i = 0; i < P->own.size() && s == LBVE_OK; ++i)
+        s = enqueue_own(P, P->own[i], nsteps, last, P->side[i % (size_t)n_own]);
+    for (int k = 0; k < nsteps && !P->batch.empty() && s == LBVE_OK; ++k)
+        s = enqueue_batch(P, q, k, last && k + 1 == nsteps);
+    if (n_own > 0) s = joined(P, s, 0, n_own);
+    if (s != LBVE_OK || n_own == 0) return s;
+    k_step_count<<<1, 1, 0, P->stream>>>(P->dstep + 1, (unsigned)nsteps);
+    PCK(cudaGetLastError(), "step counter");
     return LBVE_OK;
 }
 
@@ -1780,14 +1800,18 @@ lbve_status capture_steps(lbve_pool *P, int q, int nsteps, bool last) {
     if (exec && P->graph_steps[q][last] == nsteps) return LBVE_OK;
     if (exec) cudaGraphExecDestroy(exec);
     exec = nullptr;
-    cudaGraph_t g;
+    cudaGraph_t g = nullptr;
     PCK(cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-    lbve_status s = enqueue_steps(P, q, nsteps, last);
+    const lbve_status s = enqueue_steps(P, q, nsteps, last);
     cudaError_t e = cudaStreamEndCapture(P->stream, &g);
-    if (s != LBVE_OK) return s;
-    PCK(e, "end capture");
-    PCK(cudaGraphInstantiate(&exec, g, 0), "graph instantiate");
-    cudaGraphDestroy(g);
+    if (s == LBVE_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (s != LBVE_OK) {
+        cudaGetLastError();  // the failed capture's own error
+        return s;
+    }
+    if (e != cudaSuccess) exec = nullptr;
+    PCK(e, "graph capture");
     P->graph_steps[q][last] = nsteps;
     return LBVE_OK;
 }
@@ -1933,6 +1957,11 @@ lbve_status lbve_pool_residuals(lbve_pool *P, double *out) {
         P->res_cap = 0;
         PCK(cudaMalloc(&P->res_dev, sizeof(double) * at[n]), "residual staging");
         P->res_cap = at[n];
+    }
+    // before the fork, so that a member without memory leaves every snapshot as it is
+    for (lbve_ctx *c : P->members) {
+        const lbve_status r = residual_buffers(c);
+        if (r != LBVE_OK) return pfail(P, r, c->err);
     }
     size_t next = 0;
     lbve_status s = fan_out(P, P->members, 0, [&](lbve_ctx *c, cudaStream_t st) -> lbve_status {
