@@ -403,17 +403,20 @@ const char *lbve_noalloc_last_error(void);
 lbve_status lbve_residual(lbve_ctx *ctx, double out[2]);
 
 /*
- * Pools: resident solves that advance together.  lbve_pool_step runs each time step as
- * one persistent stream-collide kernel and one persistent stress kernel over a packed
- * list of (solve, block) work items, plus the per-solve momentum-exchange and particle
- * kernels; each cell is computed exactly as in lbve_step, so a solve's result does not
- * depend on the other members.  Members must share the pool's PDF precision and stream.
- * Admission is checked against the pool's device-memory budget (lbve_device_bytes of
- * the member's parameters); the pool never owns or frees member contexts.
- * With graphs enabled (default) the launch sequence of a step call is captured into a
- * CUDA graph and replayed while the membership and step count are unchanged (not on
- * the legacy default stream, which cannot be captured: there the kernels launch
- * directly).
+ * Pools: resident solves that advance together.  A pool that replays graphs (below) runs
+ * each member's own kernels side by side, for all members up to 64 and for those of 2^16
+ * cells and more beyond; the other members, and all of a pool without graphs, share one
+ * persistent stream-collide kernel and one persistent stress kernel per stress tile width
+ * over a packed list of (solve, block) work items, plus per-solve momentum-exchange and
+ * particle kernels.  Each cell is computed exactly as in lbve_step, so a solve's result
+ * does not depend on the other members.  Members must share the pool's PDF precision and
+ * stream.  Admission is checked against the pool's device-memory budget (lbve_device_bytes
+ * of the member's parameters); the pool never owns or frees member contexts.
+ * With graphs enabled (default) the launch sequence of a step call is captured into CUDA
+ * graphs, one of a block of steps that is replayed through the call and one of the steps
+ * that remain, and these are replayed by later calls while the membership is unchanged
+ * (the second: and the number of steps that remain).  Not on the legacy default stream,
+ * which cannot be captured: there the kernels launch directly.
  */
 typedef struct lbve_pool lbve_pool;
 lbve_status lbve_pool_create(int pdf_prec, size_t budget_bytes, void *cuda_stream, lbve_pool **out);
@@ -440,17 +443,18 @@ const char *lbve_pool_last_error(const lbve_pool *pool);
  *
  * lbve_autotune (split schedule; LBVE_ESTATE for the fused schedule or a pool member):
  * for every candidate -- stream-collide block width 32, 64 or 128 (up to the width nx
- * needs) times stress z-planes per block at half, one and two times the default --
- * `steps` untimed steps, then `steps` steps timed with CUDA events on the context's
- * stream.  The
- * fastest is kept for this context and recorded in a process-wide table keyed by
- * (precision, nx, ny, nz); contexts created later with that key start from it (unless
- * their params set block_x).  steps <= 0: apply a recorded choice only, measuring
- * nothing.  out may be NULL.
+ * needs) times stress z-planes per block at half, one and two times the default (the
+ * default only where the stress kernel has no z-chunks: FP64, and small grids under
+ * AUTO) -- `steps` untimed steps, then `steps` steps timed with CUDA events on the
+ * context's stream.  The fastest is kept for this context and recorded in a process-wide
+ * table keyed by precision, nx, ny, nz, schedule and stress update (fv_terms, Giesekus,
+ * FENE-P); contexts created later with that key start from it (unless their params set
+ * block_x).  A pool's stress kernels take their own z-chunk.  steps <= 0: apply a recorded
+ * choice only, measuring nothing.  out may be NULL.
  */
 typedef struct {
     int block_x;                 /* chosen stream-collide block width */
-    int fv_zchunk;               /* chosen stress z-planes per block */
+    int fv_zchunk;               /* chosen stress z-planes per block (1: one cell per thread) */
     int candidates;              /* schedules measured by this call */
     long long steps_taken;       /* steps the context advanced */
     double ms_per_step;          /* chosen schedule, as measured (0 if not measured) */
@@ -463,7 +467,9 @@ lbve_status lbve_autotune(lbve_ctx *ctx, int steps, lbve_tuning *out);
  * 128-thread block, up to the width nx needs) and then the stress tile width (16, 32 or
  * 64 cells of a 256-thread block; FP64: 32) are chosen by coordinate descent, each
  * candidate timed over `steps` pool steps after two untimed calls of `steps` steps (which
- * leave the step graphs of both call parities captured).  The choices are
+ * leave the step graphs of both call parities captured).  Only the batched kernels have
+ * tiles: a class whose members all have kernels of their own (see the pools above) is
+ * reported with its present widths, neither timed nor recorded.  The choices are
  * recorded per (precision, nx) and applied to contexts admitted to any pool later.  Every
  * member advances by the steps measured.  The first max_classes classes are reported
  * (arrays of max_classes entries, NULL allowed): nx, chosen tile widths; ms_before /

@@ -83,16 +83,21 @@ struct lbve_ctx {
 };
 
 namespace {
-// Process-wide record of tuned schedules: single solves by (precision, nx, ny, nz) ->
-// (stream-collide block width, stress z-planes per block); pool tiles by (precision, nx)
-// -> (stream-collide tile width, stress tile width).
+// Process-wide record of tuned schedules: single solves by tune_key -> (stream-collide
+// block width, stress z-planes per block or 0 for the default); pool tiles by (precision,
+// nx) -> (stream-collide tile width, stress tile width).
 std::mutex g_tune_mu;
-std::map<std::array<int, 4>, std::array<int, 2>> g_tuned_ctx;
+std::map<std::array<int, 6>, std::array<int, 2>> g_tuned_ctx;
 std::map<std::array<int, 2>, std::array<int, 2>> g_tuned_tiles;
 
+// What decides a solve's kernels: storage, shape, schedule and stress update.
+std::array<int, 6> tune_key(const lbve_params &p) {
+    const int law = (p.giesekus_alpha > 0.0 ? 16 : 0) + (p.fene_L2 > 0.0 ? 32 : 0);
+    return {p.pdf_prec, p.nx, p.ny, p.nz, p.schedule, p.fv_terms + law};
+}
 bool tuned_ctx(const lbve_params &p, int &bx, int &zc) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tuned_ctx.find({p.pdf_prec, p.nx, p.ny, p.nz});
+    auto it = g_tuned_ctx.find(tune_key(p));
     if (it == g_tuned_ctx.end()) return false;
     bx = it->second[0];
     zc = it->second[1];
@@ -2053,7 +2058,7 @@ lbve_status lbve_autotune(lbve_ctx *c, int steps, lbve_tuning *out) {
             c->d.fv_zchunk = zc;
         }
         r.block_x = c->d.block_x;
-        r.fv_zchunk = c->kt->fv_zchunk_of(c->d);
+        r.fv_zchunk = std::max(1, c->kt->fv_zchunk_of(c->d));
         if (out) *out = r;
         return LBVE_OK;
     }
@@ -2061,21 +2066,25 @@ lbve_status lbve_autotune(lbve_ctx *c, int steps, lbve_tuning *out) {
     const int bx0 = c->d.block_x, zc0 = c->d.fv_zchunk;
     DevState probe = c->d;
     probe.fv_zchunk = 0;
-    const int h = c->kt->fv_zchunk_of(probe);
+    const int h = c->kt->fv_zchunk_of(probe);  // 0: no stress kernel reads a chunk
     std::vector<int> bxs, zcs;
     for (int b : {32, 64, 128})
         if (b == 32 || b / 2 < c->p.nx) bxs.push_back(b);
-    for (int z : {std::max(4, h / 2), h, std::min(c->p.nz, 2 * h)})
-        if (std::find(zcs.begin(), zcs.end(), z) == zcs.end()) zcs.push_back(z);
+    if (h == 0) {
+        zcs.push_back(zc0);
+    } else {
+        for (int z : {std::max(4, h / 2), h, std::min(c->p.nz, 2 * h)})
+            if (std::find(zcs.begin(), zcs.end(), z) == zcs.end()) zcs.push_back(z);
+    }
     double ms0 = 0.0;
     lbve_status s = time_steps(c->stream, steps, 1, step, ms0, c->err);
     if (s != LBVE_OK) return s;
     double best = ms0;
-    int best_bx = bx0, best_zc = zc0 > 0 ? zc0 : h;
+    int best_bx = bx0, best_zc = zc0;  // zc0 = 0: the default chunk
     int count = 1;
     for (int b : bxs) {
         for (int z : zcs) {
-            if (b == bx0 && z == (zc0 > 0 ? zc0 : h)) continue;  // the starting schedule, measured above
+            if (b == bx0 && (h == 0 || z == (zc0 > 0 ? zc0 : h))) continue;  // the starting schedule, measured above
             c->d.block_x = b;
             c->d.fv_zchunk = z;
             double ms = 0.0;
@@ -2093,10 +2102,10 @@ lbve_status lbve_autotune(lbve_ctx *c, int steps, lbve_tuning *out) {
     c->d.fv_zchunk = best_zc;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tuned_ctx[{c->p.pdf_prec, c->p.nx, c->p.ny, c->p.nz}] = {best_bx, best_zc};
+        g_tuned_ctx[tune_key(c->p)] = {best_bx, best_zc};
     }
     r.block_x = best_bx;
-    r.fv_zchunk = best_zc;
+    r.fv_zchunk = std::max(1, c->kt->fv_zchunk_of(c->d));
     r.candidates = count;
     r.steps_taken = c->t - t0;
     r.ms_per_step = best;
@@ -2130,13 +2139,22 @@ lbve_status lbve_pool_autotune(lbve_pool *P, int steps, int max_classes, int *n_
     if (s != LBVE_OK) return s;
     double best = base;
     std::vector<std::array<int, 3>> chosen;
+    // tile widths are the batched kernels': classes whose members all have kernels of their
+    // own are reported as they are, neither timed nor recorded
+    const std::vector<lbve_ctx *> batch = P->batch;  // as the calls above built it
     for (auto &o : order) {
         const int nx = o.second;
         lbve_ctx *rep = nullptr;
+        bool tiles = false;
         for (lbve_ctx *c : P->members)
             if (c->p.nx == nx) rep = c;
+        for (lbve_ctx *c : batch) tiles |= c->p.nx == nx;
         int cur_lb = 0, cur_fv = 0;
         P->kt->batch_tiles(rep->d, rep->lb_tx, rep->fv_tx, &cur_lb, &cur_fv);
+        if (!tiles) {
+            chosen.push_back({nx, cur_lb, cur_fv});
+            continue;
+        }
         const int wmax = std::max(16, std::min(128, pow2_at_least(nx)));
         // stream-collide tile width
         for (int lb : {16, 32, 64, 128}) {

@@ -199,7 +199,8 @@ struct KernelTable {
     cudaError_t (*residual)(const DevState &, void *usnap, double *partial, int nblocks, cudaStream_t);
     // the tile widths fill_entry will use for requested widths (0: default by nx)
     void (*batch_tiles)(const DevState &, int lb_tx, int fv_tx, int *lb_eff, int *fv_eff);
-    int (*fv_zchunk_of)(const DevState &);  // z-planes per block the stress kernel will use
+    // z-planes per block the stress kernel will use, 0: the per-cell kernel, which has no chunks
+    int (*fv_zchunk_of)(const DevState &);
     int (*fv_variant_of)(const DevState &);  // 1 when the solve uses a finite-volume variant
     // pools: the particle phase of every member with particles in one launch; entries
     // built per member like the batch entries

@@ -392,7 +392,7 @@ struct Launch {
                 // per cell (256^3, FP32: two-cell 15 ps, tiled 17, per-cell 31), rows of half a
                 // column and more
                 DevState q = d;
-                q.fv_zchunk = fv_zchunk_batched(d);
+                q.fv_zchunk = fv_zchunk_batched(d);  // (a chunk tuned alone is for a chip alone)
                 if (d.g.nx >= 64 && fv_pair_shape(d)) return fv_pair(q, s);
                 if (d.g.nx >= 32) return fv_variant(d) ? fv_var<true>(q, s) : fv_var<false>(q, s);
                 return fv_cells(d, s);
@@ -542,7 +542,10 @@ struct Launch {
         *lb_items = e.lb_items;
         *fv_items = e.fv_items;
     }
-    static int fv_zchunk_of(const DevState &d) { return fv_zchunk(d); }
+    static int fv_zchunk_of(const DevState &d) {
+        if (fv_cells_ok(d)) return 0;
+        return fv_pair_ok(d) ? fv_pair_zchunk(d) : fv_zchunk(d);
+    }
     static cudaError_t lb_batched(const void *entries, int n, int total, int k, int grid, const unsigned *dstep,
                                   int parity, cudaStream_t s) {
         if (total <= 0) return cudaSuccess;
