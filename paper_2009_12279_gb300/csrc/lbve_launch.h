@@ -158,6 +158,23 @@ inline int graph_block_steps(long long nodes) {
     return (int)(steps < 2 ? 2 : steps / 2 * 2);
 }
 
+// Rows per strip of a split of ny rows on each of nz planes into n equal strips, n nz at most
+// 32 places: the split of least whole rounds of `places` blocks x (rows + 1.5).  Every launch
+// asks: only the n at which the rows change are looked at, 2 sqrt(ny) of them at most
+// (128 x 32768 x 1 cells: every n took 62 us per launch).
+inline int strip_rows(int ny, int nz, long long places) {
+    int yc = ny;
+    long long best = -1;
+    for (long long n = 1; n <= ny && (n == 1 || n * nz <= 32 * places);) {
+        const long long rows = (ny + n - 1) / n, strips = (ny + rows - 1) / rows;
+        const long long cost = (strips * nz + places - 1) / places * (2 * rows + 3);
+        if (best < 0 || cost < best) best = cost, yc = (int)rows;
+        if (rows == 1) break;
+        n = (ny + rows - 2) / (rows - 1);  // the first n with fewer rows
+    }
+    return yc;
+}
+
 struct KernelTable {
     int prec;          // lbve_pdf_prec
     size_t pdf_bytes;  // bytes per stored PDF

@@ -4,7 +4,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <climits>
 
 #include "lbve_kernels.cuh"
 #include "lbve_particles.cuh"
@@ -154,13 +153,7 @@ struct Launch {
             if (per_sm < 1) per_sm = 1;
             const long long places = sms * per_sm;
             if constexpr (sizeof(S) == 2) {
-                long long best = LLONG_MAX;
-                for (long long n = 1; n <= ny && (n == 1 || n * nzc <= 32 * places); ++n) {
-                    const int rows = (int)((ny + n - 1) / n);
-                    const long long strips = (ny + rows - 1) / rows;
-                    const long long cost = (strips * nzc + places - 1) / places * (2 * rows + 3);
-                    if (cost < best) best = cost, yc = rows;
-                }
+                yc = strip_rows(ny, nzc, places);
             } else {
                 const long long strips = std::max(1LL, (16 * places + nzc - 1) / nzc);
                 yc = std::max(8, (int)((ny + strips - 1) / strips));
@@ -358,7 +351,7 @@ struct Launch {
         int best = march_zchunk(tiles, nz, slots);
         if (best > 16 || tiles * ((nz + 15) / 16) >= 8 * slots) return best;
         double least = 0.0;
-        for (int chunks = 1; chunks <= (nz + 7) / 8; ++chunks) {
+        for (int chunks = 1; chunks <= (nz + 7) / 8;) {
             const int zc = (nz + chunks - 1) / chunks;
             const long long blocks = tiles * ((nz + zc - 1) / zc), rest = blocks % slots;
             const double t = (zc + 1.5) * (2.1 * (double)(blocks / slots) + (rest == 0 ? 0.0 : rest <= sms ? 1.3 : 2.1));
@@ -366,6 +359,8 @@ struct Launch {
                 least = t;
                 best = zc;
             }
+            if (zc == 1) break;
+            chunks = (nz + zc - 2) / (zc - 1);  // the first with fewer planes
         }
         return best;
     }
