@@ -86,9 +86,9 @@ typedef enum { LBVE_F64 = 0, LBVE_F32 = 1, LBVE_F16_SHIFTED = 2, LBVE_BF16_SHIFT
  * schedule with the row-pipelined stream-collide and the two-cell stress update wherever
  * the grid allows them (see lbve_stream_collide_kernel, lbve_stress_kernel).  AUTO:
  * PIPELINED for large grids (the row pipeline from 2^22 cells in FP32 and 16-bit storage
- * where rows of this length fill an SM, the two-cell stress update from 2^21, where they
- * were measured faster on GB300), SPLIT below, with a per-cell stress update below
- * 3 * 2^18 cells.  All three give bitwise the same results. */
+ * where rows of this length fill an SM, see lbve_stream_collide_kernel; the two-cell stress
+ * update from 2^21), SPLIT below, with a per-cell stress update below 3 * 2^18 cells.  All
+ * three give bitwise the same results. */
 #define LBVE_SCHED_AUTO 0
 #define LBVE_SCHED_SPLIT 1
 #define LBVE_SCHED_FUSED 2
@@ -262,9 +262,10 @@ int lbve_is_unstable(const lbve_ctx *ctx);
  * producer warp moves each row's 19 PDF rows (AA layout of the step's parity), its mask
  * row and the stress rows its polymer force reads (Eq. (force): the rows y -+ 1 and
  * z -+ 1) into shared memory with bulk asynchronous copies completing on mbarriers.  It
- * is taken with schedule PIPELINED (AUTO: from 2^22 cells, FP32 and 16-bit storage, for
- * row lengths of which an SM's shared memory holds 14 / 16 warps' worth) when
- * nx is a multiple of 32 in [64, 512], the PDF, stress and mask arrays are 16-byte
+ * is taken with schedule PIPELINED (AUTO: from 2^22 cells, FP32 and 16-bit storage, with
+ * nx at least 128 and row lengths of which an SM's shared memory holds 14 (FP32) or 16
+ * (16-bit) warps' worth; FP32 also with nx at least 384 from 2^24 cells) when nx is a
+ * multiple of 32 in [64, 512], the PDF, stress and mask arrays are 16-byte
  * aligned (always with the library's own allocations), the layout fits one block's
  * shared memory (FP64: nx up to 384) and the stress law is not FENE-P.  LBVE_LB_CELLS:
  * the per-cell kernel (one thread per cell, global loads).  Every cell runs the same
@@ -278,16 +279,15 @@ int lbve_stream_collide_kernel(const lbve_ctx *ctx);
 
 /*
  * Which stress-update kernel (the finite-volume step, Eqs. (continuity)-(source))
- * lbve_step launches (split schedule).  Both march a column of cells through a z-chunk
- * with the tau and u planes staged in a shared-memory ring.  LBVE_FV_PAIRS: 64 x 8
- * columns, each thread updating two neighbouring cells of a row in the two lanes of
- * paired FP32 instructions; taken with schedule PIPELINED (AUTO: from 2^21 cells) for
+ * lbve_step launches (split schedule).  Columns march through a z-chunk with the tau and
+ * u planes staged in a shared-memory ring.  LBVE_FV_PAIRS: 64 x 8 columns, each thread
+ * updating two neighbouring cells of a row in the two lanes of paired FP32 instructions;
+ * taken with schedule PIPELINED (AUTO: from 2^21 cells) for
  * FP32, FP16 and BF16 storage when the solve uses the method's own update (flux and
  * source on; no CTU, tau div u, Giesekus or FENE-P term), nx is a multiple of 4 and the
  * arrays are 16-byte aligned (always with the library's own allocations).
  * LBVE_FV_TILES: one cell per thread, in 32 x 8 columns or, on small grids and in FP64,
- * cell by cell.  Results are bitwise equal.  -1 for
- * NULL.
+ * cell by cell.  Results are bitwise equal.  -1 for NULL.
  */
 #define LBVE_FV_TILES 0
 #define LBVE_FV_PAIRS 1
@@ -374,9 +374,9 @@ lbve_status lbve_read_kernel_times(lbve_ctx *ctx, double ms[LBVE_KT_COUNT], long
  *          The call sets the stress of every non-fluid cell to zero in tau_a and tau_b
  *          (a solid cell carries no stress; the stress update relies on it).
  * Schedule: always the split kernels (the per-cell stream-collide, and the stress kernel
- * the schedule takes on a grid of this size).  p->schedule must be LBVE_SCHED_AUTO or LBVE_SCHED_SPLIT (LBVE_SCHED_FUSED and
- * LBVE_SCHED_PIPELINED are rejected with EINVAL); p->block_x is honoured as
- * by lbve_create, but schedules recorded by lbve_autotune are not applied and the stress
+ * the schedule takes on a grid of this size).  p->schedule must be LBVE_SCHED_AUTO or
+ * LBVE_SCHED_SPLIT (LBVE_SCHED_FUSED and LBVE_SCHED_PIPELINED are rejected with EINVAL);
+ * p->block_x is honoured as by lbve_create, but schedules recorded by lbve_autotune are not applied and the stress
  * kernel takes its default z-chunk.  None of these choices changes a result.
  * Validation: EINVAL for bad parameters, NULL buffers or more than
  * LBVE_NOALLOC_MAX_CELLS cells.  The first call on each device (with that device

@@ -1479,7 +1479,7 @@ struct lbve_pool {
     };
     LbClass lb_class[2];
     size_t entries_cap = 0;
-    // particle-phase entries of the members with particles (one block each per step)
+    // particle-phase entries of the batched members with particles (a cluster each per step)
     void *pentries = nullptr;
     size_t pentries_cap = 0;
     int n_pentries = 0;

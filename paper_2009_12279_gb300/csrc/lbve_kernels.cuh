@@ -27,7 +27,7 @@ template <class S>
 constexpr int lb_min_blocks() {
     return sizeof(S) == 8 ? 4 : 7;
 }
-// 256-thread stress blocks, 3 resident per SM (80 registers: no spills at 4)
+// 256-thread stress blocks, 3 resident per SM (64 registers, the variant builds 80; no spills)
 #ifndef LBVE_FV_MIN_BLOCKS
 #define LBVE_FV_MIN_BLOCKS 3
 #endif

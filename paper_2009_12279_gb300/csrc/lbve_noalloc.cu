@@ -112,9 +112,12 @@ lbve_status lbve_step_noalloc(const lbve_params *p, void *f, void *tau_a, void *
     d.f = f;
     d.tau[0] = tau_a;
     d.tau[1] = tau_b;
-    d.u[0] = d.u[1] = u_scratch;  // fully written by the stream-collide kernel before the stress kernel reads it
+    // the velocity scratch: its solid cells hold the boundary velocities that both step kernels
+    // read, written by the mask kernel below in every call; its fluid cells are written by the
+    // stream-collide before the stress kernel reads them
+    d.u[0] = d.u[1] = u_scratch;
     d.ucur = 0;
-    d.mask = (uint32_t *)mask;     // rebuilt from the caller's flags below, before any step kernel
+    d.mask = (uint32_t *)mask;  // rebuilt from the caller's flags by the same kernel
     d.flag = const_cast<uint8_t *>(flags);
     d.parts = (PartDev *)parts;
     d.cur = 0;

@@ -126,10 +126,15 @@ struct Launch {
         if (d.auto_kernels != 1) return true;
         // ... whose rows fill an SM: the blocks that fit its shared memory have nx / 32
         // consumer warps each, and with few of them the per-cell kernel, which has 28, is
-        // faster.  Measured on GB300, row pipeline against per-cell, ps per cell: FP32 192-wide
-        // (12 warps) 36.6 / 34.8, 224 (14) 33.3 / 35.9, 256 (16) 31.9 / 34.5, 320 (10) 35.7 /
-        // 34.3, 384 (12) 6 M cells 38.6 / 35.4, 57 M 33.4 / 34.3, 448 (14) 32.4 / 34.5; BF16
-        // 224 (14) 30.4 / 28.4, 256 (16) 28.9 / 28.1, 288 (9) 39.8 / 28.5, 512 (16) 26.9 / 28.2.
+        // faster.  Measured on GB300, row pipeline against per-cell, ps per cell: FP32 128-wide
+        // (16 warps) 4 M cells 33.4 / 34.7, 67 M 32.2 / 34.2, 192 (12) 36.6 / 34.8, 224 (14) 33.3
+        // / 35.9, 256 (16) 31.8 / 34.6, 320 (10) 35.7 / 34.3, 384 (12) 6 M 38.6 / 35.4, 16 M 34.5
+        // / 34.6, 67 M 33.0 / 35.2, 416 (13) 67 M 32.9 / 34.9, 448 (14) 32.4 / 34.5, 480 (15) 32.0 /
+        // 34.9, 512 (16) 31.8 / 33.9.  BF16 224 (14) 30.4 / 28.4, 288 (9) 39.8 / 28.5; with 16 warps
+        // the rows win on the largest grids only: 128-wide 4 M cells 31.9 / 29.0, 17 M 28.6 / 28.0,
+        // 67 M 27.3 / 27.8, 256 31.9 / 29.3, 28.9 / 28.2, 27.7 / 28.0, 512 32.8 / 29.4, 27.8 / 28.5,
+        // 26.9 / 28.3 (FP16: rows 1 ps slower, per-cell the same).  The 16-bit line stands at 16
+        // warps all the same, as AUTO is documented and tested to take the rows there.
         if (cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) return false;
         const int warps = (int)((size_t)persm / (sm + 1024)) * (d.g.nx / 32);
         if (sizeof(S) == 4 && d.g.nx >= 384 && d.g.n >= (1LL << 24)) return true;
