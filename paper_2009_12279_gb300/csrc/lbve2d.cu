@@ -416,7 +416,7 @@ struct lbve2d_ctx {
     double *stage = nullptr;  // FP64 staging, 15 n doubles
     void *arena = nullptr;    // the one device allocation that holds all of these but force
     // multi-step launches; here from creation on, so that lbve2d_step allocates nothing
-    unsigned *bar = nullptr;    // device word of the grid barrier
+    unsigned *bar = nullptr;    // device: the grid barrier's two words
     unsigned *stuck = nullptr;  // mapped host word: 2 once a barrier's bounded wait gave up
     unsigned *stuck_dev = nullptr;
     int resident = -1;          // tiles the device holds at once (-1: not asked yet)
@@ -606,7 +606,7 @@ lbve_status lbve2d_create(const lbve2d_params *p, void *cuda_stream, lbve2d_ctx 
     const size_t at_f[2] = {take(Q2 * n * c->rb), take(Q2 * n * c->rb)};
     const size_t at_tau[2] = {take(3 * n * c->rb), take(3 * n * c->rb)};
     const size_t at_u = take(2 * n * c->rb), at_ub = take(2 * n * c->rb), at_flag = take(n);
-    const size_t at_stage = take(15 * n * sizeof(double)), at_bar = take(sizeof(unsigned));
+    const size_t at_stage = take(15 * n * sizeof(double)), at_bar = take(2 * sizeof(unsigned));
     cudaError_t e = cudaMalloc(&c->arena, bytes);
     if (e == cudaSuccess) {
         char *p0 = (char *)c->arena;
@@ -700,6 +700,7 @@ lbve_status lbve2d_init_fields(lbve2d_ctx *c, const double *rho, const double *u
     if (u) CK2(cudaMemcpyAsync(su, u, sizeof(double) * 2 * n, cudaMemcpyHostToDevice, c->stream), "init copy");
     if (tau) CK2(cudaMemcpyAsync(stau, tau, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, c->stream), "init copy");
     c->cur = 0;
+    CK2(cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream), "barrier reset");
     const unsigned nb = (unsigned)((n + 255) / 256);
     if (c->rb == 8) {
         Args2<double> a = args2<double>(c);

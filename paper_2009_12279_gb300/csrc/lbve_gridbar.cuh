@@ -27,11 +27,12 @@ inline int launch_steps(int steps, long long blocks) {
     return (int)std::min<long long>(steps, std::max(1LL, most));
 }
 
-// Barrier number k (0, 1, ...) of `blocks` blocks on a word that was 0 at the launch's start:
+// Barrier number k (0, 1, ...) of `blocks` blocks on word[0], which was 0 at the launch's start:
 // they count up to (k + 1) blocks, at most 2^30 (launch_steps).  False (in every thread of
-// the block) when the wait gave up, after writing 2 to *status and marking the word, or when
-// another block did: the caller returns then, and so do the others, at this barrier or the
-// next.  The block barriers around the release add and the acquire load make every thread's
+// the block) when the wait gave up, after writing 2 to *status, 1 to word[1] and marking
+// word[0], or when another block did: the caller returns then, and so do the others, at this
+// barrier or the next.  While word[1] stays set the first barrier of a launch returns false
+// at once, so that the launches of a long call do not each wait in turn.  The block barriers around the release add and the acquire load make every thread's
 // earlier writes visible to every thread's later reads (PTX causality order); fences of their
 // own would only add to it.
 __device__ __forceinline__ bool grid_barrier(unsigned *word, unsigned k, unsigned blocks, unsigned *status,
@@ -44,8 +45,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *word, unsigned k, unsigne
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
         const unsigned long long limit = k == 0 ? first_ns : wait_ns;
         unsigned long long t0 = 0;
-        ok = 1;
-        for (unsigned n = 0;; ++n) {
+        const unsigned given_up = k == 0 ? *(volatile const unsigned *)(word + 1) : 0u;
+        ok = given_up == 0u;
+        for (unsigned n = 0; given_up == 0u; ++n) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
             if (v >= target) {
@@ -59,6 +61,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *word, unsigned k, unsigne
                     t0 = t;
                 else if (t - t0 > limit) {
                     atomicOr(word, GB_LEFT);
+                    *(volatile unsigned *)(word + 1) = 1u;
                     if (status) *(volatile unsigned *)status = 2u;
                     ok = 0;
                     break;

@@ -14,24 +14,25 @@ pytestmark = pytest.mark.gpu
 
 SRC = """
 #include "lbve_gridbar.cuh"
-// Blocks of 64 threads meet `steps` times on word out[0]; out[1] is the status word, out[2 + b]
-// becomes the number of barriers block b passed.  Block 0 waits at most first_ns0 at the
+// Blocks of 64 threads meet `steps` times on the words out[0..1]; out[2] is the status word,
+// out[3 + b] becomes the number of barriers block b passed.  Block 0 waits at most first_ns0 at the
 // first barrier, the others first_ns.
 __global__ void k_meet(unsigned *out, int steps, unsigned blocks, unsigned long long first_ns0,
                        unsigned long long first_ns, unsigned long long wait_ns) {
     unsigned passed = 0;
     for (int s = 0; s < steps; ++s) {
-        if (!lbve::grid_barrier(out, (unsigned)s, blocks, out + 1, blockIdx.x == 0 ? first_ns0 : first_ns, wait_ns)) break;
+        if (!lbve::grid_barrier(out, (unsigned)s, blocks, out + 2, blockIdx.x == 0 ? first_ns0 : first_ns, wait_ns)) break;
         ++passed;
     }
-    if (threadIdx.x == 0) out[2 + blockIdx.x] = passed;
+    if (threadIdx.x == 0) out[3 + blockIdx.x] = passed;
 }
 extern "C" int meet(unsigned *host, int nblocks, int steps, unsigned blocks, unsigned long long first_ns0,
                     unsigned long long first_ns, unsigned long long wait_ns) {
     unsigned *d = nullptr;
-    const size_t bytes = sizeof(unsigned) * (2 + (size_t)nblocks);
+    const size_t bytes = sizeof(unsigned) * (3 + (size_t)nblocks);
     if (cudaMalloc((void **)&d, bytes) != cudaSuccess) return -1;
     cudaError_t e = cudaMemset(d, 0, bytes);
+    if (e == cudaSuccess) e = cudaMemcpy(d + 1, host + 1, sizeof(unsigned), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         void *args[] = {&d, &steps, &blocks, &first_ns0, &first_ns, &wait_ns};
         e = cudaLaunchCooperativeKernel((const void *)k_meet, dim3(nblocks), dim3(64), args, 0, nullptr);
@@ -59,11 +60,13 @@ def meet(tmp_path_factory):
     u64 = ctypes.c_ulonglong
     lib.meet.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_uint, u64, u64, u64]
 
-    def call(nblocks, steps, blocks, first0, first, wait):
-        out = (ctypes.c_uint * (2 + nblocks))()
+    def call(nblocks, steps, blocks, first0, first, wait, given_up=0):
+        out = (ctypes.c_uint * (3 + nblocks))()
+        out[1] = given_up
         t = time.monotonic()
         assert lib.meet(out, nblocks, steps, blocks, first0, first, wait) == 0
-        return out[0], out[1], list(out[2:]), time.monotonic() - t
+        assert out[1] == (1 if given_up or out[2] else 0)
+        return out[0], out[2], list(out[3:]), time.monotonic() - t
 
     return call
 
@@ -78,6 +81,13 @@ def test_every_block_passes_every_barrier(meet, nblocks, steps):
 def test_a_wait_that_runs_out_sets_the_status(meet, nblocks):
     word, status, passed, _ = meet(nblocks, 4, nblocks + 1, 20 * MS, 20 * MS, 20 * MS)
     assert status == 2 and passed == [0] * nblocks and word >> 31 == 1
+
+
+def test_no_wait_after_a_launch_that_gave_up(meet):
+    """The second word still set: the launches behind one that gave up return at once."""
+    meet(1, 1, 1, MS, MS, MS)
+    word, status, passed, seconds = meet(64, 4, 65, 5000 * MS, 5000 * MS, 20 * MS, given_up=1)
+    assert status == 0 and passed == [0] * 64 and seconds < 2.5
 
 
 def test_one_block_that_gives_up_ends_the_waits_of_the_others(meet):
