@@ -1924,10 +1924,10 @@ lbve_status lbve_pool_step(lbve_pool *P, int nsteps) {
     }
     const int q = (int)(P->steps_since_build & 1);
     if (pool_graphs(P)) {
-        // A call longer than a block of graph_block_steps() steps replays a graph of that many
+        // A call longer than a block of graph_block_steps steps replays a graph of that many
         // (an even number: parities and ping-pongs return to where they were) and ends with
         // one of the remaining 1 to block steps, which includes the forces on wall classes.
-        const int block = graph_block_steps(step_nodes(P)), blocks = (nsteps - 1) / block;
+        const int block = graph_block_steps(step_nodes(P), nsteps), blocks = (nsteps - 1) / block;
         lbve_status s = blocks > 0 ? capture_steps(P, q, block, false) : LBVE_OK;
         if (s == LBVE_OK) s = capture_steps(P, q, nsteps - blocks * block, true);
         if (s != LBVE_OK) return s;

@@ -146,16 +146,26 @@ inline cudaError_t launch_step(int pdl, void (*kernel)(P...), dim3 grid, dim3 bl
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
-// Steps of a pool's replayed graph, an even number, for steps of `nodes` kernels each: about
-// GRAPH_NODES kernels to capture, instantiate and keep, however long a call is.  48 members of
-// the serving mix, BF16, ms of the first call after an admission and of a replay: 100 steps in
-// one graph 113 / 68.2, blocks of 1024 kernels 72 / 68.3, 2048 75 / 68.0, 4096 83 / 68.2, 8192
-// 114 / 68.0; 1000 steps 1198 / 687 (402 MB on the device), 690 / 684, 691 / 679 (55 MB), 704 /
-// 683, 736 / 684.
-constexpr long long GRAPH_NODES = 2048;
-inline int graph_block_steps(long long nodes) {
-    const long long steps = GRAPH_NODES / (nodes > 0 ? nodes : 1);
-    return (int)(steps < 2 ? 2 : steps / 2 * 2);
+// Steps of a pool's replayed graph, an even number, for steps of `nodes` kernels each: at most
+// about GRAPH_NODES kernels to capture, instantiate and keep, however long a call is.  A call
+// of more steps than the longest block takes the block of at least half of it that leaves the
+// fewest steps to capture (100 steps, at most 30: six blocks of 16 and four steps).  48 members
+// of the serving mix, some 130 kernels a step, BF16, ms of the first call after an admission
+// and of a replay: 25 steps in one graph 27.0 / 16.9; with blocks of at most 1024, 2048 and 4096
+// kernels 20.0 / 17.0, 21.3 / 17.0 and 27.7 / 16.8 (one graph); 100 steps 111 / 68.0; 71.9 / 68.3,
+// 73.5 / 67.6, 75.8 / 67.9; 1000 steps 1201 / 686 (402 MB on the device); 692 / 684, 690 / 679,
+// 692 / 679 (54 MB).
+constexpr long long GRAPH_NODES = 4096;
+inline int graph_block_steps(long long nodes, int nsteps) {
+    const long long fit = GRAPH_NODES / (nodes > 0 ? nodes : 1);
+    const int most = fit < 2 ? 2 : (int)(fit / 2 * 2);
+    if (nsteps <= most) return most;
+    int best = most, least = most + (nsteps - 1) % most + 1;
+    for (int b = most - 2; b >= 2 && 2 * b >= most; b -= 2) {
+        const int captured = b + (nsteps - 1) % b + 1;
+        if (captured < least) best = b, least = captured;
+    }
+    return best;
 }
 
 // Rows per strip of a split of ny rows on each of nz planes into n equal strips, n nz at most
