@@ -71,6 +71,7 @@ struct lbve_ctx {
     long long kt_count[LBVE_KT_COUNT] = {0};
     // steady-state residual
     void *usnap = nullptr;
+    bool usnap_clear = false;  // the snapshot is new and has to be set to zero
     double *res_partial = nullptr;
     lbve_pool *pool = nullptr;
     // instability flag: mapped page-locked word set by the stream-collide (d.bad is its
@@ -1382,23 +1383,26 @@ static int residual_blocks(const lbve_ctx *c) {
 // The residual's buffers, made by the first call: all of them or none.
 static lbve_status residual_buffers(lbve_ctx *c) {
     if (c->usnap) return LBVE_OK;
-    const size_t bytes = (size_t)3 * c->d.g.np * c->kt->real_bytes;
-    void *snap = dev_alloc(c, bytes);
+    void *snap = dev_alloc(c, (size_t)3 * c->d.g.np * c->kt->real_bytes);
     double *partial = (double *)dev_alloc(c, sizeof(double) * 2 * 1024);
-    const cudaError_t e = snap && partial ? cudaMemsetAsync(snap, 0, bytes, c->stream) : cudaSuccess;
-    if (!snap || !partial || e != cudaSuccess) {
+    if (!snap || !partial) {
         dev_free(c, snap);
         dev_free(c, partial);
-        CK(e, "residual clear");
         return fail(c, LBVE_ENOMEM, "residual buffers");
     }
     c->usnap = snap;
     c->res_partial = partial;
+    c->usnap_clear = true;
     return LBVE_OK;
 }
 
-// Block partials of the residual into `partial`, on a stream that follows the context's.
+// Block partials of the residual into `partial`, on a stream that follows the context's; the
+// first time the snapshot is cleared there, too.
 static lbve_status residual_enqueue(lbve_ctx *c, double *partial, cudaStream_t st) {
+    if (c->usnap_clear) {
+        CK(cudaMemsetAsync(c->usnap, 0, (size_t)3 * c->d.g.np * c->kt->real_bytes, st), "residual clear");
+        c->usnap_clear = false;
+    }
     CK(c->kt->residual(c->d, c->usnap, partial, residual_blocks(c), st), "residual kernel");
     return LBVE_OK;
 }
